@@ -70,7 +70,7 @@ template <int TS, int RPT, int C, bool BF16, bool TSRC>
 constexpr size_t bilinear_bwd_smem() {
     constexpr int D = TS * TS * RPT;
     return sizeof(uint32_t) * stages_for<TS, RPT>() * D * bwd_ring_stride<C, BF16, TSRC>()  // record ring
-           + sizeof(float) * 4 * 2 * D                                              // (T a, w dL/da) per slot
+           + sizeof(float2) * 4 * D                                                 // (T a, w dL/da) per parity
            + sizeof(float) * TS * TS * C                                            // upstream dL/dF per pixel
            + 128;
 }
@@ -104,17 +104,16 @@ __global__ void __launch_bounds__(TS * TS, TS == 8 && RPT == 1 ? 16 : 1) k_blend
     constexpr int FW = RecLayout<0, C, BF16>::feat_word;
     extern __shared__ __align__(128) uint32_t s_dyn[];
     uint32_t* const s_ring = align128(s_dyn);                                 // [kStages][D][RS]
-    float* const s_ta = reinterpret_cast<float*>(s_ring + kStages * D * RS);  // [4][D]
-    float* const s_da = s_ta + 4 * D;                                         // [4][D]
-    float* const s_gF = s_da + 4 * D;                                         // [NT][C]
+    float2* const s_td = reinterpret_cast<float2*>(s_ring + kStages * D * RS);  // [4][D] (T a, w dL/da)
+    float* const s_gF = reinterpret_cast<float*>(s_td + 4 * D);                 // [NT][C]
     __shared__ uint32_t s_mask[NT][MW + 1];
-    // Per record: the bilinear weights and the 1 / (1 - alpha) of its 2x2
-    // slots, and (tile-local anchor, depth bits, opacity bits). A fragment
-    // reads the three with independent vector loads and picks its slot in
-    // registers, so no shared-memory load waits on another one.
-    __shared__ float4 s_w4[D];
-    __shared__ float4 s_inv4[D];
-    __shared__ uint4 s_azo[D];
+    // Per record: the bilinear weight and the 1 / (1 - alpha) of each pixel of
+    // its 2x2 box, indexed by the pixel's parity (x & 1) + 2 (y & 1), and its
+    // (opacity, depth). A 2x2 box holds each parity once, so a pixel's pair is
+    // at an offset that is fixed for the thread (no anchor to compare), and the
+    // contributions it leaves for the record's thread are filed the same way.
+    __shared__ float4 s_wi[D][2];
+    __shared__ float2 s_oz[D];
     __shared__ uint32_t s_red;
     __shared__ __align__(8) uint64_t s_mbar[kStages];  // TSRC: one bulk-copy barrier per ring stage
 
@@ -128,6 +127,9 @@ __global__ void __launch_bounds__(TS * TS, TS == 8 && RPT == 1 ? 16 : 1) k_blend
     const bool inside = px < V.W && py < V.H;
     const uint2 rg = ranges[tile];
     const float amax = vt.alpha_max;
+    const int parity = (lx & 1) | ((ly & 1) << 1);
+    const float2* const my_wi = reinterpret_cast<const float2*>(s_wi) + parity;
+    float2* const my_td = s_td + parity * D;
 
     float T = 1.f, Tfin = 1.f, gA = 0.f, gD = 0.f;
     float gF[C];
@@ -228,10 +230,7 @@ __global__ void __launch_bounds__(TS * TS, TS == 8 && RPT == 1 ? 16 : 1) k_blend
         const uint32_t* ring = s_ring + (size_t)st * D * RS;
         const uint32_t rel0 = bi * D;
 #pragma unroll
-        for (int k = 0; k < 4 * RPT; ++k) {
-            s_ta[k * NT + tid] = 0.f;
-            s_da[k * NT + tid] = 0.f;
-        }
+        for (int k = 0; k < 4 * RPT; ++k) s_td[k * NT + tid] = make_float2(0.f, 0.f);
         if (bulk) {
             if (mbar_wait(&s_mbar[st], (phase >> st) & 1u)) {
                 phase ^= 1u << st;
@@ -261,17 +260,19 @@ __global__ void __launch_bounds__(TS * TS, TS == 8 && RPT == 1 ? 16 : 1) k_blend
             const BilinGeom bg = bilin_geom(__uint_as_float(g.x), __uint_as_float(g.y));
             const float o = __uint_as_float(g.w);
             const float ax = __fsub_rn(1.f, bg.a), by = __fsub_rn(1.f, bg.b);
-            const float w0 = __fmul_rn(ax, by), w1 = __fmul_rn(bg.a, by);
-            const float w2 = __fmul_rn(ax, bg.b), w3 = __fmul_rn(bg.a, bg.b);
-            s_w4[r] = make_float4(w0, w1, w2, w3);
-            // 1 / (1 - alpha) of each slot, alpha = min(o w, amax) exactly as the forward has it
-            s_inv4[r] = make_float4(rcp_fast(__fsub_rn(1.f, fminf(__fmul_rn(o, w0), amax))),
-                                    rcp_fast(__fsub_rn(1.f, fminf(__fmul_rn(o, w1), amax))),
-                                    rcp_fast(__fsub_rn(1.f, fminf(__fmul_rn(o, w2), amax))),
-                                    rcp_fast(__fsub_rn(1.f, fminf(__fmul_rn(o, w3), amax))));
             const int X0 = bg.i0 - tx * TS, Y0 = bg.j0 - ty * TS;
+            // weights of the even and the odd column and row of the box
+            const float we = (X0 & 1) ? bg.a : ax, wo = (X0 & 1) ? ax : bg.a;
+            const float he = (Y0 & 1) ? bg.b : by, ho = (Y0 & 1) ? by : bg.b;
+            const float w0 = __fmul_rn(we, he), w1 = __fmul_rn(wo, he);
+            const float w2 = __fmul_rn(we, ho), w3 = __fmul_rn(wo, ho);
+            // 1 / (1 - alpha), alpha = min(o w, amax) exactly as the forward has it
+            s_wi[r][0] = make_float4(w0, rcp_fast(__fsub_rn(1.f, fminf(__fmul_rn(o, w0), amax))),
+                                     w1, rcp_fast(__fsub_rn(1.f, fminf(__fmul_rn(o, w1), amax))));
+            s_wi[r][1] = make_float4(w2, rcp_fast(__fsub_rn(1.f, fminf(__fmul_rn(o, w2), amax))),
+                                     w3, rcp_fast(__fsub_rn(1.f, fminf(__fmul_rn(o, w3), amax))));
+            s_oz[r] = make_float2(o, __uint_as_float(g.z));
             anchor[k] = (X0 + 1) | ((Y0 + 1) << 8);
-            s_azo[r] = make_uint4((uint32_t)anchor[k], g.z, g.w, 0u);
             const uint32_t bit = 1u << lane;
             const int word = r >> 5;
 #pragma unroll
@@ -312,14 +313,10 @@ __global__ void __launch_bounds__(TS * TS, TS == 8 && RPT == 1 ? 16 : 1) k_blend
                 m &= ~(1u << bit);
                 const int r = w * 32 + bit;
                 if (rel0 + r >= last) continue;
-                const uint4 azo = s_azo[r];
-                const float4 w4 = s_w4[r];
-                const float4 i4 = s_inv4[r];
-                const bool sx = lx + 1 != (int)(azo.x & 0xffu), sy = ly + 1 != (int)(azo.x >> 8);
-                const int slot = (int)sx + 2 * (int)sy;
-                const float wgt = sy ? (sx ? w4.w : w4.z) : (sx ? w4.y : w4.x);
-                const float inv = sy ? (sx ? i4.w : i4.z) : (sx ? i4.y : i4.x);
-                const float ow = __fmul_rn(__uint_as_float(azo.z), wgt);
+                const float2 wi = my_wi[4 * r];
+                const float2 oz = s_oz[r];
+                const float wgt = wi.x, inv = wi.y, z = oz.y;
+                const float ow = __fmul_rn(oz.x, wgt);
                 const float alpha = fminf(ow, amax);
                 const float Tk = T * inv;  // T_k = T_{k+1} / (1 - alpha_k)
                 const uint32_t* rp = ring + r * RS;
@@ -328,14 +325,12 @@ __global__ void __launch_bounds__(TS * TS, TS == 8 && RPT == 1 ? 16 : 1) k_blend
                 float fdot = 0.f;
 #pragma unroll
                 for (int c = 0; c < C; ++c) fdot = fmaf(gF[c], f[c], fdot);
-                const float z = __uint_as_float(azo.y);
                 const float dalpha = Tk * (fdot + gD * z) - (Sg + gD * SD + Kd) * inv;
                 const float ta = Tk * alpha;
                 Sg = fmaf(ta, fdot, Sg);
                 SD = fmaf(ta, z, SD);
                 T = Tk;
-                s_ta[slot * D + r] = ta;
-                s_da[slot * D + r] = (ow <= amax) ? wgt * dalpha : 0.f;
+                my_td[r] = make_float2(ta, (ow <= amax) ? wgt * dalpha : 0.f);
             }
         }
 #pragma unroll
@@ -372,13 +367,14 @@ __global__ void __launch_bounds__(TS * TS, TS == 8 && RPT == 1 ? 16 : 1) k_blend
 #pragma unroll
             for (int sl = 0; sl < 4; ++sl) {
                 const int X = X0 + (sl & 1), Y = Y0 + (sl >> 1);
-                const float ta = s_ta[sl * D + r];
+                const float2 td = s_td[((X & 1) + 2 * (Y & 1)) * D + r];
+                const float ta = td.x;
                 if ((unsigned)X < (unsigned)TS && (unsigned)Y < (unsigned)TS) {
                     const float* gp = s_gF + (Y * TS + X) * C;
 #pragma unroll
                     for (int c = 0; c < C; ++c) acc[c] += ta * gp[c];
                 }
-                acc[C] += s_da[sl * D + r];
+                acc[C] += td.y;
             }
             if (single[k]) {
                 if constexpr (direct_feat_grads(C, TS)) {

@@ -123,12 +123,12 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_bilinear(
     extern __shared__ __align__(128) uint32_t s_dyn[];
     uint32_t* const s_ring = align128(s_dyn);  // [kStages][D][RS] raw records
     __shared__ uint32_t s_mask[NT][MW + 1];    // MW words + 1 pad: conflict-free row reads
-    // Per record: the alphas of its 2x2 slots (FP32, pinned ops) and (tile-local
-    // anchor (X0 + 1) | (Y0 + 1) << 8, depth bits). A fragment reads both with
-    // two independent vector loads and picks its slot's alpha in registers, so
-    // no shared-memory load waits on another one.
+    // Per record: the alphas of its 2x2 box (FP32, pinned ops), indexed by the
+    // parity (x & 1) + 2 (y & 1) of the covered pixel, and its depth. A 2x2 box
+    // holds each parity once, so a pixel finds its own alpha at an offset that
+    // is fixed for the thread: one 4-byte load, with no anchor to compare.
     __shared__ float4 s_alpha4[D];
-    __shared__ uint2 s_az[D];
+    __shared__ float s_z[D];
     __shared__ uint32_t s_maxstop;
 
     const int64_t tile = order[blockIdx.x];
@@ -143,6 +143,7 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_bilinear(
     const uint32_t len = rg.y - rg.x;
     const uint32_t nbatch = (len + D - 1) / D;
     const float amax = vt.alpha_max, tmin = vt.t_min;
+    const float* const my_alpha = reinterpret_cast<const float*>(s_alpha4) + ((lx & 1) | ((ly & 1) << 1));
 
     float T = 1.f, A = 0.f, Dp = 0.f;
     float F[C];
@@ -212,12 +213,15 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_bilinear(
                 const BilinGeom bg = bilin_geom(__uint_as_float(g.x), __uint_as_float(g.y));
                 const float o = __uint_as_float(g.w);
                 const float ax = __fsub_rn(1.f, bg.a), by = __fsub_rn(1.f, bg.b);
-                s_alpha4[r] = make_float4(fminf(__fmul_rn(o, __fmul_rn(ax, by)), amax),
-                                          fminf(__fmul_rn(o, __fmul_rn(bg.a, by)), amax),
-                                          fminf(__fmul_rn(o, __fmul_rn(ax, bg.b)), amax),
-                                          fminf(__fmul_rn(o, __fmul_rn(bg.a, bg.b)), amax));
                 const int X0 = bg.i0 - tx * TS, Y0 = bg.j0 - ty * TS;
-                s_az[r] = make_uint2((uint32_t)(X0 + 1) | ((uint32_t)(Y0 + 1) << 8), g.z);
+                // weights of the even and the odd column and row of the box
+                const float we = (X0 & 1) ? bg.a : ax, wo = (X0 & 1) ? ax : bg.a;
+                const float he = (Y0 & 1) ? bg.b : by, ho = (Y0 & 1) ? by : bg.b;
+                s_alpha4[r] = make_float4(fminf(__fmul_rn(o, __fmul_rn(we, he)), amax),
+                                          fminf(__fmul_rn(o, __fmul_rn(wo, he)), amax),
+                                          fminf(__fmul_rn(o, __fmul_rn(we, ho)), amax),
+                                          fminf(__fmul_rn(o, __fmul_rn(wo, ho)), amax));
+                s_z[r] = __uint_as_float(g.z);
                 const uint32_t bit = 1u << lane;
                 const int word = r >> 5;
 #pragma unroll
@@ -243,10 +247,8 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_bilinear(
                 if (m == 0) break;
                 const int r = w * 32 + __ffs(m) - 1;
                 m &= m - 1;
-                const uint2 az = s_az[r];
-                const float4 a4 = s_alpha4[r];
-                const bool sx = lx + 1 != (int)(az.x & 0xffu), sy = ly + 1 != (int)(az.x >> 8);
-                const float alpha = sy ? (sx ? a4.w : a4.z) : (sx ? a4.y : a4.x);
+                const float alpha = my_alpha[4 * r];
+                const float z = s_z[r];
                 const float nT = __fmul_rn(T, __fsub_rn(1.f, alpha));
                 if (nT < tmin) {
                     done = true;
@@ -259,7 +261,7 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_bilinear(
                 const float ta = T * alpha;
 #pragma unroll
                 for (int c = 0; c < C; ++c) F[c] = fmaf(ta, f[c], F[c]);
-                Dp = fmaf(ta, __uint_as_float(az.y), Dp);
+                Dp = fmaf(ta, z, Dp);
                 A += ta;
                 T = nT;
                 last = rel0 + r + 1;
