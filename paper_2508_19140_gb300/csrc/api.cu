@@ -61,6 +61,7 @@ struct Plan {
     size_t bytes[S_COUNT];
     size_t total;
     int64_t copy_cap, blk_cap;
+    int64_t expectA, expectC;  // elements the two sorts are expected to have (their launch shapes)
     SortPlan planA, planC;
     int partial_floats;
     int arrangement;
@@ -253,12 +254,23 @@ rast_status_t make_plan(const rast_view_t* views, int32_t n_views, const rast_op
     pl.bytes[S_GROW] = o->mode == RAST_SPLAT_BILINEAR ? (size_t)N * grow_stride(C + 1) * 4 : 0;
     pl.bytes[S_SGHIST] = (size_t)kMaxSortPasses * 512 * 4;
     pl.bytes[S_SCOUNT] = (size_t)kMaxSortPasses * 4;
+    int64_t sort_words;
     {
         // The 64-bit-key arrangement sorts copies, not points, by depth.
         const int64_t na = arrangement == kUntiledKey64 ? pl.copy_cap : npt;
-        const int64_t wa = sort_status_words(pl.planA, na), wc = sort_status_words(pl.planC, pl.copy_cap);
-        pl.bytes[S_SSTATUS] = (size_t)(wa > wc ? wa : wc) * 4;
+        // Copies a point makes, as the launch shapes assume them: about 1.25 (bilinear
+        // tiles), 2 (small Gaussians), 4 (one-pixel tiles).
+        const int64_t ec = untiled ? 4 * npt : (o->mode == RAST_SPLAT_BILINEAR ? npt + npt / 4 : 2 * npt);
+        pl.expectC = ec < pl.copy_cap ? ec : pl.copy_cap;
+        pl.expectA = arrangement == kUntiledKey64 ? pl.expectC : npt;
+        const int64_t wa = sort_status_words(pl.planA, na, pl.expectA);
+        const int64_t wc = sort_status_words(pl.planC, pl.copy_cap, pl.expectC);
+        sort_words = wa > wc ? wa : wc;
     }
+    // The sorts' look-back words live where the backward's partial rows will
+    // (no sort runs in a backward pass, no partial row outlives one).
+    pl.bytes[S_SSTATUS] = 0;
+    if (pl.bytes[S_PARTIAL] < (size_t)sort_words * 4) pl.bytes[S_PARTIAL] = (size_t)sort_words * 4;
     pl.bytes[S_PIXC] = pl.bytes[S_PTC] = arrangement == kUntiledKey64 ? (size_t)D * 4 : 0;
     // Bilinear tiled: the forward blend writes every record it reads, in
     // tile-list order, so the backward reads its batches sequentially.
@@ -311,7 +323,7 @@ Bufs make_bufs(const Plan& pl, void* ws) {
     b.grow = (float*)at(S_GROW);
     b.sort_ghist = (uint32_t*)at(S_SGHIST);
     b.sort_counters = (uint32_t*)at(S_SCOUNT);
-    b.sort_status = (uint32_t*)at(S_SSTATUS);
+    b.sort_status = (uint32_t*)at(S_PARTIAL);
     b.ranges = (uint2*)at(S_RANGES);
     b.order = (uint32_t*)at(S_ORDER);
     b.cutoff = (uint2*)at(S_CUTOFF);
@@ -427,7 +439,7 @@ cudaError_t run_fwd(const Plan& pl, const Bufs& b, cudaStream_t s) {
         const SortScratch sc{b.sort_ghist, b.sort_counters, b.sort_status, &b.hdr->error,
                              (vt.flags & RAST_FLAG_TEST_SORT_STALL) != 0};
         // Only the depth order of the point indices is used after this sort.
-        RAST_TRY(radix_sort(k, v, vt.n_total, nullptr, vt.n_total, pl.planA, sc, s, &ra, kDepthSortNames,
+        RAST_TRY(radix_sort(k, v, vt.n_total, nullptr, vt.n_total, pl.expectA, pl.planA, sc, s, &ra, kDepthSortNames,
                             true, false));
     }
     const uint32_t* depth_sorted = b.valA[ra];
@@ -438,7 +450,7 @@ cudaError_t run_fwd(const Plan& pl, const Bufs& b, cudaStream_t s) {
         uint32_t* k[2] = {b.keyC[0], b.keyC[1]};
         uint32_t* v[2] = {b.valC[0], b.valC[1]};
         const SortScratch sc{b.sort_ghist, b.sort_counters, b.sort_status, &b.hdr->error};
-        RAST_TRY(radix_sort(k, v, 0, &b.hdr->n_copies, pl.copy_cap, pl.planC, sc, s, &rc, kTileSortNames));
+        RAST_TRY(radix_sort(k, v, 0, &b.hdr->n_copies, pl.copy_cap, pl.expectC, pl.planC, sc, s, &rc, kTileSortNames));
     }
     RAST_TRY(launch_ranges(vt, b, b.keyC[rc], s));
     if (vt.tile == 1) return launch_blend_fwd_pixel(vt, b, b.valC[rc], s);  // untiled baseline
@@ -482,7 +494,7 @@ cudaError_t run_fwd_key64(const Plan& pl, const Bufs& b, cudaStream_t s) {
         uint32_t* k[2] = {b.keyC[0], b.keyC[1]};
         uint32_t* v[2] = {b.valC[0], b.valC[1]};
         // Low word: the values are the copy ids (generated by the first pass).
-        RAST_TRY(radix_sort(k, v, 0, &b.hdr->n_copies, pl.copy_cap, pl.planA, sc, s, &ra, kLoNames, true, false));
+        RAST_TRY(radix_sort(k, v, 0, &b.hdr->n_copies, pl.copy_cap, pl.expectA, pl.planA, sc, s, &ra, kLoNames, true, false));
     }
     const int g = ra ^ 1;
     RAST_TRY(launch_gather_hi(b, b.valC[ra], b.pixC, b.ptC, b.keyC[g], b.valC[g], s));
@@ -491,7 +503,7 @@ cudaError_t run_fwd_key64(const Plan& pl, const Bufs& b, cudaStream_t s) {
         uint32_t* v[2] = {b.valC[g], b.valC[ra]};
         SortScratch sc2 = sc;
         sc2.stall_test = false;
-        RAST_TRY(radix_sort(k, v, 0, &b.hdr->n_copies, pl.copy_cap, pl.planC, sc2, s, &rb, kHiNames));
+        RAST_TRY(radix_sort(k, v, 0, &b.hdr->n_copies, pl.copy_cap, pl.expectC, pl.planC, sc2, s, &rb, kHiNames));
     }
     const int r = key64_result_pair(pl);
     RAST_TRY(launch_ranges(vt, b, b.keyC[r], s));

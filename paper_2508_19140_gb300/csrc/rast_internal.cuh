@@ -263,8 +263,9 @@ struct SortPlan {
     int shift[8];
 };
 SortPlan make_sort_plan(int bits);
-// Look-back words one sort with this plan needs for `cap` elements.
-int64_t sort_status_words(const SortPlan& plan, int64_t cap);
+// Look-back words one sort with this plan needs for `cap` elements, launched
+// for about `expect` of them.
+int64_t sort_status_words(const SortPlan& plan, int64_t cap, int64_t expect);
 
 struct SortScratch {
     uint32_t* ghist;     // [kMaxSortPasses][512]
@@ -278,14 +279,14 @@ struct SortScratch {
 // when the depth sort makes no pass).
 cudaError_t launch_project(const ViewTable& vt, const Bufs& b, bool write_vals, cudaStream_t s);
 // Stable LSD radix sort of (key, val) pairs in keys[0]/vals[0] using keys[1]/vals[1]
-// as scratch; count from d_n (device) if non-null else n (at most cap). Sets
-// *result_buf to the index (0/1) of the buffer that holds the result.
+// as scratch; count from d_n (device) if non-null else n (at most cap); expect:
+// the count the launch shapes are chosen for. Sets *result_buf to the index (0/1) of the buffer that holds the result.
 // names: profiling names of the digit-count kernel and of the sweep passes.
 // identity_vals: the input values are their own positions (0, 1, 2, ...);
 // vals[0] is then not read. keys_out = false: only the values are wanted, the
 // last pass does not write keys (keys[*result_buf] is left stale).
 cudaError_t radix_sort(uint32_t* keys[2], uint32_t* vals[2], int64_t n, const uint32_t* d_n, int64_t cap,
-                       const SortPlan& plan, const SortScratch& sc, cudaStream_t s, int* result_buf,
+                       int64_t expect, const SortPlan& plan, const SortScratch& sc, cudaStream_t s, int* result_buf,
                        const char* const names[2], bool identity_vals = false, bool keys_out = true);
 cudaError_t launch_duplicate(const ViewTable& vt, const Bufs& b, const uint32_t* sorted_pts,
                              cudaStream_t s);

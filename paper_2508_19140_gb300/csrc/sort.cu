@@ -10,36 +10,42 @@
 //   k_digit_hist  one read of all keys counts the digits of every pass at once
 //                 (digit counts do not depend on the order), and clears the
 //                 per-pass tile counters and look-back status words;
-//   k_sweep       per pass, persistent CTAs take 4096-key tiles in input order
-//                 from an atomic counter, rank each key stably inside the tile
-//                 (one ballot per digit bit, or one match instruction for
-//                 9-bit digits, gives each lane the mask of lanes holding the
-//                 same digit; warps counted in ascending order),
-//                 publish the tile's per-digit counts, and add the counts of
-//                 all earlier tiles by looking back over their published words
-//                 eight at a time (a tile whose whole prefix is known publishes
-//                 it, so walks are short). Keys are then staged in shared
-//                 memory in digit order and written out in runs.
+//   k_sweep       per pass, persistent CTAs take tiles of 256 * IPT keys in
+//                 input order from an atomic counter; keys and values arrive by
+//                 bulk copies. Each warp counts the digits of its own keys in
+//                 shared memory (one increment a key), the tile's counts are
+//                 published, and the warps' counters become the tile-local
+//                 start of every (digit, warp). A key's place in the tile is
+//                 then its digit's running counter plus the number of lower
+//                 lanes with the same digit, and key and value go to shared
+//                 memory there at once. After the threads have looked back for
+//                 the counts of all earlier tiles, both leave shared memory in
+//                 digit order, in runs.
+// Look-back in two levels: a tile publishes its counts on their own and adds
+// them to its group's sums (kGroup tiles; the word also counts the arrivals),
+// and the group's last tile publishes the inclusive prefix. A tile sums the
+// tiles before it in its group (one round of loads) and walks back over whole
+// groups, so hundreds of tiles that start together wait on a few round trips
+// rather than on a chain through all of them.
 // A tile only waits on tiles that running CTAs took before it, so the waits
 // always end; each wait is still bounded, and on expiry the kernel raises the
 // timeout bit of the workspace error word and carries on with the partial
 // prefix instead of spinning on. The element count may live on the device (copies
-// are counted on the GPU): launch shapes depend only on the capacity.
-#include <cuda/atomic>
-
-#include "rast_internal.cuh"
+// are counted on the GPU): launch shapes depend only on the capacity and on
+// the count the caller expects.
+#include "blend_common.cuh"
 
 namespace rast {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kIPT = 16;
-constexpr int kSortTile = kThreads * kIPT;  // 4096 keys per tile
-constexpr int kWarpItems = 32 * kIPT;       // 512 keys per warp
-constexpr uint32_t kFlagAgg = 1u << 30;     // tile count published
-constexpr uint32_t kFlagPrefix = 2u << 30;  // inclusive prefix over tiles 0..t published
+constexpr int kWarps = kThreads / 32;
+constexpr int kGroup = 16;                  // tiles per look-back group
+constexpr int kGroupWindow = 8;             // groups read per look-back step
+constexpr uint32_t kFlag = 1u << 31;        // word published (tile counts, group prefixes)
 constexpr uint32_t kValueMask = (1u << 30) - 1;
-constexpr int kLookback = 8;               // predecessor tiles read per look-back step
+constexpr uint32_t kArrival = 1u << 24;     // group sums: one arrival; the sum (at most kGroup tiles) below it
+static_assert(kGroup * kThreads * 16 < (1 << 24) && kGroup < 128, "group sums and arrivals share a word");
 
 __device__ __forceinline__ int64_t read_count(int64_t n_host, const uint32_t* d_n) {
     return d_n ? (int64_t)(*d_n) : n_host;
@@ -79,6 +85,22 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t x, uint32_t* s_warp
     return res;
 }
 
+// Look-back words of one pass: per tile its digit counts, then per group the
+// (inclusive prefix, sum and arrivals) pairs. A single tile has none.
+struct StatusLayout {
+    int64_t tiles, groups;
+    int64_t pass_words;  // words of one pass
+};
+template <int BITS>
+__host__ __device__ inline StatusLayout status_layout(int64_t cap, int tile_keys) {
+    StatusLayout l;
+    l.tiles = (cap + tile_keys - 1) / tile_keys;
+    if (l.tiles == 1) l.tiles = 0;
+    l.groups = (l.tiles + kGroup - 1) / kGroup;
+    l.pass_words = (l.tiles + 2 * l.groups) << BITS;
+    return l;
+}
+
 // Digit counts of every pass with one read of the keys; clears the tile
 // counters and the look-back words the passes will use.
 template <int BITS>
@@ -86,18 +108,21 @@ __global__ void __launch_bounds__(kThreads) k_digit_hist(const uint32_t* __restr
                                                          const uint32_t* d_n, int passes,
                                                          uint32_t* __restrict__ ghist,
                                                          uint32_t* __restrict__ counters,
-                                                         uint32_t* __restrict__ status, int64_t tiles_cap) {
+                                                         uint32_t* __restrict__ status, int64_t cap, int tile_keys) {
     constexpr int BINS = 1 << BITS;
     __shared__ uint32_t s_h[kMaxSortPasses * BINS];
     const int64_t n = read_count(n_host, d_n);
-    const int64_t ntiles = (n + kSortTile - 1) / kSortTile;
     for (int i = threadIdx.x; i < passes * BINS; i += kThreads) s_h[i] = 0;
     if (blockIdx.x == 0 && threadIdx.x < kMaxSortPasses) counters[threadIdx.x] = 0;
-    for (int p = 0; p < passes; ++p) {
-        uint32_t* st = status + (int64_t)p * tiles_cap * BINS;
-        const int64_t words = ntiles * BINS;
-        for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < words; i += (int64_t)gridDim.x * kThreads)
-            st[i] = 0;
+    {
+        const StatusLayout full = status_layout<BITS>(cap, tile_keys), used = status_layout<BITS>(n, tile_keys);
+        const int64_t t0 = (int64_t)blockIdx.x * kThreads + threadIdx.x, dt = (int64_t)gridDim.x * kThreads;
+        for (int p = 0; p < passes; ++p) {
+            uint32_t* st = status + p * full.pass_words;
+            for (int64_t i = t0; i < used.tiles << BITS; i += dt) st[i] = 0;
+            uint32_t* gr = st + (full.tiles << BITS);
+            for (int64_t i = t0; i < (2 * used.groups) << BITS; i += dt) gr[i] = 0;
+        }
     }
     __syncthreads();
     // Eight independent loads in flight per thread before the shared-memory
@@ -123,43 +148,168 @@ __global__ void __launch_bounds__(kThreads) k_digit_hist(const uint32_t* __restr
         if (s_h[i]) atomicAdd(&ghist[i], s_h[i]);
 }
 
+__device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ uint2 ld_relaxed2(const uint2* p) {
+    uint2 v;
+    asm volatile("ld.relaxed.gpu.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void st_relaxed(uint32_t* p, uint32_t v) {
+    asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+// Counts of one digit over all tiles before `tile` (look-back). status points
+// at the digit's word of tile 0, groups at its pair of group 0; rows are BINS
+// apart. The words of the tiles before it in its group and of the nearest
+// groups are read in one round; whole groups are then added nearest first
+// until one has its inclusive prefix. Gives up after `limit` polls: the
+// partial sum, with *err raised.
+template <int BINS>
+__device__ __forceinline__ uint32_t look_back(int64_t tile, const uint32_t* status, const uint2* groups,
+                                              uint32_t limit, uint32_t* err) {
+    const int left = (int)(tile & (kGroup - 1));
+    const uint32_t* st = status + (tile - left) * BINS;
+    int64_t q = tile / kGroup - 1;  // next group to add
+    uint32_t spins = 0, sum = 0, own = 0;
+    bool own_done = left == 0;
+    for (;;) {
+        uint32_t w[kGroup - 1];
+        uint2 g[kGroupWindow];
+        if (!own_done) {
+#pragma unroll
+            for (int j = 0; j < kGroup - 1; ++j) w[j] = j < left ? ld_relaxed(st + j * BINS) : kFlag;
+        }
+        if (q >= 0) {
+#pragma unroll
+            for (int j = 0; j < kGroupWindow; ++j)
+                g[j] = q - j >= 0 ? ld_relaxed2(groups + (q - j) * BINS) : make_uint2(kFlag, 0u);
+        }
+        bool waits = false;  // a word that is not there yet
+        if (!own_done) {
+            uint32_t all = kFlag;
+            own = 0;
+#pragma unroll
+            for (int j = 0; j < kGroup - 1; ++j) {
+                all &= w[j];
+                own += w[j] & kValueMask;
+            }
+            own_done = all != 0u;
+            waits = !own_done;
+        }
+        if (q >= 0) {
+            bool open = true;
+#pragma unroll
+            for (int j = 0; j < kGroupWindow; ++j) {
+                if (!open) continue;
+                if (g[j].x & kFlag) {
+                    sum += g[j].x & kValueMask;
+                    q = -1;
+                    open = false;
+                } else if (g[j].y >= kGroup * kArrival) {
+                    sum += g[j].y & (kArrival - 1);
+                    --q;
+                } else {
+                    waits = true;
+                    open = false;
+                }
+            }
+        }
+        if (own_done && q < 0) return sum + own;
+        if (waits) {
+            if (++spins > limit) {
+                atomicOr(err, kErrTimeout);
+                return sum + own;
+            }
+            __nanosleep(20);
+        }
+    }
+}
+
+template <int BITS, int IPT>
+constexpr size_t sweep_smem() {
+    return 128 + sizeof(uint32_t) * (3 * kThreads * IPT + (2 * kWarps + 2) * (1 << BITS));
+}
+
 // IDV: the input values are their positions (not read from memory).
-template <int BITS, bool IDV>
-__global__ void __launch_bounds__(kThreads, 3) k_sweep(
+//
+// Tiles arrive by TMA bulk copies, one for the keys and one for the values,
+// into three shared buffers that change roles from tile to tile: the keys are
+// read into registers and sorted in place, the values go from their buffer to
+// the spare one, the next tile's keys are fetched into the emptied values
+// buffer while this tile is written out, and its values into the spare one
+// after that. No thread holds values or waits on a global load.
+//
+// Bound by the shared-memory pipe (about one wavefront a key: counting, ranking
+// and scattering by digit; 75 % of its cycles on 32 M keys), then by the integer
+// pipe. The ranking takes the lane masks of every other round from ballots
+// (integer pipe) and of the rounds between from a shared atomic OR (memory
+// pipe): all rounds from ballots were 172 us, all from the OR 159 us, both in
+// turn 151 us a pass over 32 M keys. Three CTAs on an SM (80 registers, 57 KB)
+// with the next tile on its way beat four without: 147 us. The whole pass went
+// 217 -> 147 us (32 M keys, 7-bit digits; 3.6 TB/s moved), 36.6 -> 27 us (4 M
+// keys), 433 -> 308 us (62 M keys, 8-bit), 630 -> 535 us (77 M keys, 9-bit).
+template <int BITS, int IPT, bool IDV>
+__global__ void __launch_bounds__(kThreads, IPT == 16 ? 3 : 4) k_sweep(
     const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint32_t* __restrict__ kout,
-    uint32_t* __restrict__ vout, int64_t n_host, const uint32_t* d_n, int shift,
+    uint32_t* __restrict__ vout, int64_t n_host, const uint32_t* d_n, int64_t cap, int shift,
     const uint32_t* __restrict__ ghist_pass, uint32_t* __restrict__ counter, uint32_t* __restrict__ status,
     uint32_t* __restrict__ err, int stall_test) {
     constexpr int BINS = 1 << BITS;
-    constexpr int VPT = BINS > kThreads ? BINS / kThreads : 1;
-    extern __shared__ uint32_t smem[];
-    uint32_t* s_keys = smem;                       // kSortTile: keys in digit order
-    uint32_t* s_vals = s_keys + kSortTile;         // kSortTile: values in digit order
-    uint32_t* s_vin = s_vals + kSortTile;          // kSortTile: values in input order
-    uint32_t* s_whist = s_vin + kSortTile;         // 8 * BINS: per-warp counts, then prefixes
-    uint32_t* s_excl = s_whist + 8 * BINS;         // BINS: tile-local digit starts
-    uint32_t* s_gbase = s_excl + BINS;             // BINS: global digit starts of this tile
-    uint32_t* s_goff = s_gbase + BINS;             // BINS: global digit starts of the pass
-    uint32_t* s_thist = s_goff + BINS;             // BINS: the tile's digit counts
-    uint32_t* s_warp = s_thist + BINS;             // 33
-    uint32_t* s_tile = s_warp + 33;                // 1
+    constexpr int VPT = BINS > kThreads ? BINS / kThreads : 1;  // consecutive bins per thread
+    constexpr int TILE = kThreads * IPT;
+    extern __shared__ __align__(128) uint32_t s_dyn[];
+    uint32_t* s_k = align128(s_dyn);  // TILE: the tile's keys, then its keys in digit order
+    uint32_t* s_v = s_k + TILE;       // TILE: the tile's values, then the next tile's keys
+    uint32_t* s_s = s_v + TILE;       // TILE: values in digit order, then the next tile's values
+    uint2* const s_tab = reinterpret_cast<uint2*>(s_s + TILE);  // kWarps * BINS: (lanes, count, then running position)
+    uint32_t* const s_goff = reinterpret_cast<uint32_t*>(s_tab + kWarps * BINS);  // BINS: global digit starts
+    uint32_t* const s_ofs = s_goff + BINS;                      // BINS: global minus tile-local digit start
+    __shared__ uint32_t s_warp[33];
+    __shared__ uint32_t s_tile;
+    __shared__ __align__(8) uint64_t s_mbar[2];  // keys arrived, values arrived
     // A pass after one whose look-back wait ran out does nothing: its input
     // is a partial order whose digit counts no longer match the histogram,
     // so its scatter positions could leave the buffers. (Within the pass that
     // gave up, a partial prefix only lowers positions: they stay in [0, n).)
-    if (*err & kErrTimeout) return;
+    if (__syncthreads_or((*err & kErrTimeout) != 0u)) return;
     const int64_t n = read_count(n_host, d_n);
-    const int64_t ntiles = (n + kSortTile - 1) / kSortTile;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t ntiles = (n + TILE - 1) / TILE;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t lt = lanemask_lt();
+    uint2* const groups = reinterpret_cast<uint2*>(status + (status_layout<BITS>(cap, TILE).tiles << BITS));
+    uint2* const tab = s_tab + warp * BINS;
+    const int w0 = warp * (32 * IPT) + lane;  // this lane's first key in a tile
 
+    // One bulk copy of tile t's words (rounded up to 16 bytes: the arrays are
+    // padded to 256), by thread 0.
+    auto fetch = [&](uint32_t* dst, const uint32_t* src, int64_t t, uint64_t* bar) {
+        const int64_t left = n - t * TILE;
+        const uint32_t words = ((uint32_t)(left < TILE ? left : TILE) + 3u) & ~3u;
+        bulk_copy_g2s(dst, src + t * TILE, words * 4u, bar);
+    };
+    if (tid == 0) {
+        mbar_init(&s_mbar[0], 1);
+        mbar_init(&s_mbar[1], 1);
+        mbar_init_fence();
+        s_tile = atomicAdd(counter, 1u);
+        if (s_tile < ntiles) {
+            fetch(s_k, kin, s_tile, &s_mbar[0]);
+            if (!IDV) fetch(s_v, vin, s_tile, &s_mbar[1]);
+        }
+    }
     // Global start of every digit in this pass.
     {
         uint32_t tot[VPT];
         uint32_t local = 0;
 #pragma unroll
         for (int q = 0; q < VPT; ++q) {
-            const int bin = threadIdx.x * VPT + q;
+            const int bin = tid * VPT + q;
             tot[q] = bin < BINS ? ghist_pass[bin] : 0u;
             local += tot[q];
         }
@@ -167,246 +317,214 @@ __global__ void __launch_bounds__(kThreads, 3) k_sweep(
         uint32_t ex = block_excl_scan<kThreads>(local, s_warp, all);
 #pragma unroll
         for (int q = 0; q < VPT; ++q) {
-            const int bin = threadIdx.x * VPT + q;
+            const int bin = tid * VPT + q;
             if (bin < BINS) s_goff[bin] = ex;
             ex += tot[q];
         }
     }
-
-    // The next tile is taken from the counter during the previous tile's last
-    // phase, so the loop spends no barrier on it. (A CTA holds the next tile
-    // only while finishing one it took earlier, which never waits on it: every
-    // look-back still ends.)
-    for (int i = threadIdx.x; i < BINS; i += kThreads) s_thist[i] = 0;
-    if (threadIdx.x == 0) *s_tile = atomicAdd(counter, 1u);
     __syncthreads();
-    for (;;) {
-        const int64_t tile = *s_tile;
-        if (tile >= ntiles) break;
-        const int64_t base = tile * kSortTile;
-        const int64_t wbase = base + warp * kWarpItems;
-        // Keys to registers; values straight to shared memory in input order
-        // (they are only moved, never inspected).
-        uint32_t k[kIPT];
+    int64_t tile = s_tile;
+    uint32_t phase = 0;
+    const uint32_t limit = stall_test ? 64u : (1u << 22);
+    while (tile < ntiles) {
+        const int64_t base = tile * TILE;
+        const int cnt = (int)(n - base < TILE ? n - base : TILE);
+        // The next tile is taken now, its keys are fetched while this one is
+        // written out. (Every wait is on tiles taken earlier, whose counts are
+        // published before any wait of theirs: the look-backs still end.)
+        uint32_t next = 0;
+        if (tid == 0) next = atomicAdd(counter, 1u);
 #pragma unroll
-        for (int r = 0; r < kIPT; ++r) {
-            const int64_t idx = wbase + r * 32 + lane;
-            const bool ok = idx < n;
-            k[r] = ok ? kin[idx] : 0u;
-            s_vin[warp * kWarpItems + r * 32 + lane] = ok ? (IDV ? (uint32_t)idx : vin[idx]) : 0u;
+        for (int i = 0; i < (BINS + 31) / 32; ++i)
+            if (i * 32 + lane < BINS) tab[i * 32 + lane] = make_uint2(0u, 0u);
+        bool failed = !mbar_wait(&s_mbar[0], phase);
+        // Keys past the end are all ones: they have the highest digit and come
+        // last in input order, so they rank behind every real key.
+        uint32_t k[IPT];
+        if (cnt == TILE) {
+#pragma unroll
+            for (int r = 0; r < IPT; ++r) k[r] = s_k[w0 + r * 32];
+        } else {
+#pragma unroll
+            for (int r = 0; r < IPT; ++r) k[r] = w0 + r * 32 < cnt ? s_k[w0 + r * 32] : 0xffffffffu;
         }
-        // The tile's digit counts first (shared-memory adds), so they are
-        // published before the ranking: a successor's look-back then rarely
-        // finds this tile unpublished.
+        __syncwarp();
 #pragma unroll
-        for (int r = 0; r < kIPT; ++r)
-            if (wbase + r * 32 + lane < n) atomicAdd(&s_thist[(k[r] >> shift) & (BINS - 1)], 1u);
-        for (int i = threadIdx.x; i < 8 * BINS; i += kThreads) s_whist[i] = 0;
-        __syncthreads();
-        // Publish the tile's counts (test hook: with stall_test the first
-        // tile publishes nothing, so its successor's wait runs out).
-        uint32_t* my = status + tile * BINS;
-        const bool withhold = stall_test && tile == 0;
-        const uint32_t spin_limit = stall_test ? 64u : (1u << 22);
+        for (int r = 0; r < IPT; ++r) atomicAdd(&tab[(k[r] >> shift) & (BINS - 1)].y, 1u);
+        if (__syncthreads_or(failed)) {  // a copy never arrived: report it, let the other land, stop
+            if (tid == 0) atomicOr(err, kErrTimeout);
+            mbar_wait(&s_mbar[0], phase);
+            if (!IDV) mbar_wait(&s_mbar[1], phase);
+            break;
+        }
+
+        // Publish the tile's counts (test hook: with stall_test the first tile
+        // publishes nothing, so its successor's wait runs out), and turn the
+        // warps' counts into tile-local positions (digit, then warp).
+        const bool publish = ntiles > 1 && !(stall_test && tile == 0);
+        uint32_t tot[VPT];           // the tile's count of this thread's bins, keys past the end left out
+        uint32_t c[VPT][kWarps];     // each warp's count
+        uint32_t local = 0;          // all of them
 #pragma unroll
         for (int q = 0; q < VPT; ++q) {
-            const int bin = threadIdx.x * VPT + q;
-            if (bin < BINS && !withhold) {
-                cuda::atomic_ref<uint32_t, cuda::thread_scope_device> w(my[bin]);
-                w.store((tile == 0 ? kFlagPrefix : kFlagAgg) | s_thist[bin], cuda::memory_order_relaxed);
+            const int bin = tid * VPT + q;
+            uint32_t sum = 0;
+            if (bin < BINS) {
+#pragma unroll
+                for (int w = 0; w < kWarps; ++w) {
+                    c[q][w] = s_tab[w * BINS + bin].y;
+                    sum += c[q][w];
+                }
+                tot[q] = sum - (bin == BINS - 1 ? (uint32_t)(TILE - cnt) : 0u);
+                if (publish) {
+                    st_relaxed(status + tile * BINS + bin, kFlag | tot[q]);
+                    atomicAdd(&groups[(tile / kGroup) * BINS + bin].y, kArrival | tot[q]);
+                }
+            }
+            local += sum;
+        }
+        const uint32_t inc = warp_incl_scan(local);
+        if (lane == 31) s_warp[warp] = inc;
+        __syncthreads();
+        uint32_t run = inc - local;
+#pragma unroll
+        for (int w = 0; w < kWarps - 1; ++w) run += w < warp ? s_warp[w] : 0u;
+        uint32_t start[VPT];
+#pragma unroll
+        for (int q = 0; q < VPT; ++q) {
+            const int bin = tid * VPT + q;
+            start[q] = run;
+            if (bin < BINS) {
+#pragma unroll
+                for (int w = 0; w < kWarps; ++w) {
+                    s_tab[w * BINS + bin].y = run;
+                    run += c[q][w];
+                }
             }
         }
+        if (!IDV) failed = !mbar_wait(&s_mbar[1], phase);
+        if (__syncthreads_or(failed)) {
+            if (tid == 0) atomicOr(err, kErrTimeout);
+            mbar_wait(&s_mbar[1], phase);
+            break;
+        }
+        phase ^= 1u;
 
-        // Stable rank inside the warp's 512 keys: rounds in input order, lanes
-        // in order within a round. Ranks (< 512) are kept two to a register.
-        uint32_t lp[kIPT / 2];
+        // Stable rank: rounds in input order, lanes in order within a round.
 #pragma unroll
-        for (int r = 0; r < kIPT / 2; ++r) lp[r] = 0;
-#pragma unroll
-        for (int r = 0; r < kIPT; ++r) {
-            const int64_t idx = wbase + r * 32 + lane;
-            const bool ok = idx < n;
-            const uint32_t d = ok ? ((k[r] >> shift) & (BINS - 1)) : 0u;
-            // Lanes holding the same digit. Up to 8-bit digits: one ballot per
-            // digit bit (and one for validity); 9-bit digits: one match
-            // instruction, measured faster there (lanes past the end share a
-            // digit value of their own).
-            uint32_t peers;
-            if constexpr (BITS >= 9) {
-                peers = __match_any_sync(0xffffffffu, ok ? d : (uint32_t)BINS);
-            } else {
-                peers = __ballot_sync(0xffffffffu, ok);
-                if (!ok) peers = ~peers;
+        for (int r = 0; r < IPT; ++r) {
+            const uint32_t d = (k[r] >> shift) & (BINS - 1);
+            uint32_t peers, pre;  // lanes holding the same digit; the digit's next position
+            if (r & 1) {
+                peers = 0xffffffffu;
 #pragma unroll
                 for (int bb = 0; bb < BITS; ++bb) {
                     const bool set = (d >> bb) & 1u;
                     const uint32_t m = __ballot_sync(0xffffffffu, set);
                     peers &= set ? m : ~m;
                 }
+                pre = tab[d].y;
+            } else {
+                atomicOr(&tab[d].x, 1u << lane);
+                __syncwarp();
+                const uint2 t = tab[d];
+                peers = t.x;
+                pre = t.y;
             }
-            // The first lane of each digit group adds the group to the warp's
-            // counter (atomics of one warp to one address apply in program
-            // order, so rounds need no barrier) and hands the old value on.
-            const int leader = __ffs(peers) - 1;
-            uint32_t pre = 0;
-            if (ok && lane == leader) pre = atomicAdd(&s_whist[warp * BINS + d], (uint32_t)__popc(peers));
-            pre = __shfl_sync(0xffffffffu, pre, leader);
-            lp[r >> 1] |= (pre + __popc(peers & lt)) << ((r & 1) * 16);
-        }
-        __syncthreads();
-
-        // Per digit: warp prefixes (ascending warp = ascending input order) and
-        // the tile's count.
-        uint32_t tot[VPT];
-#pragma unroll
-        for (int q = 0; q < VPT; ++q) {
-            const int bin = threadIdx.x * VPT + q;
-            uint32_t run = 0;
-            if (bin < BINS) {
-#pragma unroll
-                for (int w = 0; w < 8; ++w) {
-                    const uint32_t c = s_whist[w * BINS + bin];
-                    s_whist[w * BINS + bin] = run;
-                    run += c;
-                }
-            }
-            tot[q] = run;
-        }
-        // Look back for the counts of all earlier tiles and publish the
-        // inclusive prefix.
-#pragma unroll
-        for (int q = 0; q < VPT; ++q) {
-            const int bin = threadIdx.x * VPT + q;
-            if (bin < BINS) s_excl[bin] = tot[q];  // tile-local digit counts, scanned in place below
-        }
-        __syncthreads();
-        // Tile-local digit starts: warp 0 scans the BINS counts in place (each
-        // lane a run of consecutive bins) while the other warps look back.
-        if (warp == 0) {
-            constexpr int PER = BINS >= 32 ? BINS / 32 : 1;
-            uint32_t c[PER], sum = 0;
-#pragma unroll
-            for (int q = 0; q < PER; ++q) {
-                const int bin = lane * PER + q;
-                c[q] = bin < BINS ? s_excl[bin] : 0u;
-                sum += c[q];
-            }
-            uint32_t run = warp_incl_scan(sum) - sum;
-#pragma unroll
-            for (int q = 0; q < PER; ++q) {
-                const int bin = lane * PER + q;
-                if (bin < BINS) s_excl[bin] = run;
-                run += c[q];
-            }
+            const uint32_t below = __popc(peers & lt);
+            __syncwarp();
+            if (below == 0) tab[d] = make_uint2(0u, pre + __popc(peers));
+            __syncwarp();
+            s_k[pre + below] = k[r];
+            s_s[pre + below] = IDV ? (uint32_t)base + (uint32_t)(w0 + r * 32) : s_v[w0 + r * 32];
         }
 #pragma unroll
         for (int q = 0; q < VPT; ++q) {
-            const int bin = threadIdx.x * VPT + q;
+            const int bin = tid * VPT + q;
             if (bin >= BINS) continue;
-            // Look back over windows of kLookback predecessors: the window's
-            // loads are independent and in flight together, so a walk over
-            // many tiles that only published their own counts costs one load
-            // latency per window instead of one per tile.
-            uint32_t excl = 0;
-            int64_t t = tile - 1;
-            uint32_t spins = 0;
-            while (t >= 0) {
-                uint32_t w[kLookback];
-#pragma unroll
-                for (int j = 0; j < kLookback; ++j) {
-                    w[j] = kFlagPrefix;  // before tile 0: an empty prefix
-                    if (t - j >= 0) {
-                        cuda::atomic_ref<uint32_t, cuda::thread_scope_device> a(status[(t - j) * BINS + bin]);
-                        w[j] = a.load(cuda::memory_order_relaxed);
-                    }
-                }
-                int j = 0;
-                bool found = false;
-                for (; j < kLookback; ++j) {
-                    if ((w[j] >> 30) == 0u) break;  // not published yet: poll again from here
-                    excl += w[j] & kValueMask;
-                    if ((w[j] & kFlagPrefix) != 0u) {
-                        found = true;
-                        break;
-                    }
-                }
-                if (found) break;
-                t -= j;
-                if (j < kLookback) {
-                    if (++spins > spin_limit) {  // a predecessor never published: give up
-                        atomicOr(err, kErrTimeout);
-                        break;
-                    }
-                    __nanosleep(64);
-                }
-            }
-            if (tile != 0) {
-                cuda::atomic_ref<uint32_t, cuda::thread_scope_device> w(my[bin]);
-                w.store(kFlagPrefix | (excl + tot[q]), cuda::memory_order_relaxed);
-            }
-            s_gbase[bin] = s_goff[bin] + excl;
+            const uint32_t excl = look_back<BINS>(tile, status + bin, groups + bin, limit, err);
+            if ((tile & (kGroup - 1)) == kGroup - 1)  // more than one tile
+                st_relaxed(&groups[(tile / kGroup) * BINS + bin].x, kFlag | (excl + tot[q]));
+            s_ofs[bin] = s_goff[bin] + excl - start[q];
         }
+        if (tid == 0) s_tile = next;
+        fence_proxy_async();  // this thread's accesses to the buffers come before the copies into them
         __syncthreads();
+        tile = s_tile;
+        if (tid == 0 && tile < ntiles) fetch(s_v, kin, tile, &s_mbar[0]);
 
+        if (cnt == TILE) {
+            constexpr int U = 4;
+#pragma unroll 1
+            for (int j0 = tid; j0 < TILE; j0 += U * kThreads) {
+                uint32_t key[U], val[U], dst[U];
 #pragma unroll
-        for (int r = 0; r < kIPT; ++r) {
-            const int64_t idx = wbase + r * 32 + lane;
-            if (idx < n) {
-                const uint32_t d = (k[r] >> shift) & (BINS - 1);
-                const uint32_t rank = (lp[r >> 1] >> ((r & 1) * 16)) & 0xffffu;
-                const uint32_t pos = s_excl[d] + s_whist[warp * BINS + d] + rank;
-                s_keys[pos] = k[r];
-                s_vals[pos] = s_vin[warp * kWarpItems + r * 32 + lane];
+                for (int u = 0; u < U; ++u) {
+                    key[u] = s_k[j0 + u * kThreads];
+                    val[u] = s_s[j0 + u * kThreads];
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    dst[u] = s_ofs[(key[u] >> shift) & (BINS - 1)] + (uint32_t)(j0 + u * kThreads);
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (kout) kout[dst[u]] = key[u];
+                    vout[dst[u]] = val[u];
+                }
+            }
+        } else {
+            for (int j = tid; j < cnt; j += kThreads) {
+                const uint32_t key = s_k[j];
+                const uint32_t dst = s_ofs[(key >> shift) & (BINS - 1)] + (uint32_t)j;
+                if (kout) kout[dst] = key;
+                vout[dst] = s_s[j];
             }
         }
-        __syncthreads();
-
-        const int cntv = (int)(n - base < kSortTile ? n - base : kSortTile);
-        for (int j = threadIdx.x; j < cntv; j += kThreads) {
-            const uint32_t key = s_keys[j];
-            const uint32_t d = (key >> shift) & (BINS - 1);
-            const uint32_t dst = s_gbase[d] + ((uint32_t)j - s_excl[d]);
-            if (kout) kout[dst] = key;
-            vout[dst] = s_vals[j];
-        }
-        for (int i = threadIdx.x; i < BINS; i += kThreads) s_thist[i] = 0;  // read before the look-back barrier
-        if (threadIdx.x == 0) *s_tile = atomicAdd(counter, 1u);  // every thread has read this tile's index
-        __syncthreads();
+        fence_proxy_async();
+        __syncthreads();  // the tile's keys, values and offsets are read
+        if (!IDV && tid == 0 && tile < ntiles) fetch(s_s, vin, tile, &s_mbar[1]);
+        uint32_t* const free_buf = s_k;
+        s_k = s_v;
+        s_v = s_s;
+        s_s = free_buf;
     }
 }
 
-template <int BITS>
-size_t sweep_smem() {
-    constexpr int BINS = 1 << BITS;
-    return sizeof(uint32_t) * (3 * kSortTile + 8 * BINS + 4 * BINS + 33 + 1);
-}
+// Keys per thread of the sweeps, by the count a sort is expected to have: tiles
+// of 4096 keys, which spend the least on counts and look-back (4 M points 27.3
+// us a pass, with 1024-key tiles 42.3 us; 500 k points 10.8 against 12.8 us),
+// unless so few keys would occupy only a part of the SMs (20 k points 8.7
+// against 10.1 us, 60 k points 9.3 against 10.4 us).
+int sweep_ipt(int64_t expect) { return expect <= 256 * 1024 ? 4 : 16; }
 
-template <int BITS>
+template <int BITS, int IPT>
 cudaError_t sort_t(uint32_t* keys[2], uint32_t* vals[2], int64_t n, const uint32_t* d_n, int64_t cap,
                    const SortPlan& plan, const SortScratch& sc, cudaStream_t s, int* result_buf,
                    const char* const names[2], bool identity_vals, bool keys_out) {
     constexpr int BINS = 1 << BITS;
+    constexpr int TILE = kThreads * IPT;
     // Launch attributes and the resident CTAs per SM of the sweep, once per
     // device: persistent grid = as many CTAs as fit on the GPU at once (every
     // CTA resident, so a look-back never waits on a tile no running CTA holds).
     static PerDevice setup;
-    const size_t smem = sweep_smem<BITS>();
+    constexpr size_t smem = sweep_smem<BITS, IPT>();
     int per_sm = 1;
-    cudaError_t e = per_device(setup, &per_sm, [smem](int, int* v) {
+    cudaError_t e = per_device(setup, &per_sm, [](int, int* v) {
         *v = 1;
-        cudaError_t r =
-            cudaFuncSetAttribute(k_sweep<BITS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t r = cudaFuncSetAttribute(k_sweep<BITS, IPT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)smem);
         if (r == cudaSuccess)
-            r = cudaFuncSetAttribute(k_sweep<BITS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            r = cudaFuncSetAttribute(k_sweep<BITS, IPT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)smem);
         if (r != cudaSuccess) return r;
         int occ = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_sweep<BITS, false>, kThreads, smem) ==
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_sweep<BITS, IPT, false>, kThreads, smem) ==
                 cudaSuccess && occ >= 1)
             *v = occ;
         return cudaSuccess;
     });
     if (e != cudaSuccess) return e;
-    const int64_t tiles_cap = (cap + kSortTile - 1) / kSortTile;
+    const StatusLayout sl = status_layout<BITS>(cap, TILE);
     const int sms = device_sm_count();
     e = cudaMemsetAsync(sc.ghist, 0, sizeof(uint32_t) * plan.passes * BINS, s);
     if (e != cudaSuccess) return e;
@@ -416,27 +534,37 @@ cudaError_t sort_t(uint32_t* keys[2], uint32_t* vals[2], int64_t n, const uint32
         if (g > (int64_t)sms * 4) g = (int64_t)sms * 4;
         if (g < 1) g = 1;
         k_digit_hist<BITS><<<(unsigned)g, kThreads, 0, s>>>(keys[0], n, d_n, plan.passes, sc.ghist,
-                                                           sc.counters, sc.status, tiles_cap);
+                                                           sc.counters, sc.status, cap, TILE);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     const int64_t resident = (int64_t)sms * per_sm;
-    const unsigned gs = (unsigned)(tiles_cap < resident ? tiles_cap : resident);
+    const int64_t tiles = sl.tiles > 0 ? sl.tiles : 1;
+    const unsigned gs = (unsigned)(tiles < resident ? tiles : resident);
     int cur = 0;
     for (int k = 0; k < plan.passes; ++k) {
         ProfScope ps(names[1], s);
-        auto kern = (k == 0 && identity_vals) ? k_sweep<BITS, true> : k_sweep<BITS, false>;
+        auto kern = (k == 0 && identity_vals) ? k_sweep<BITS, IPT, true> : k_sweep<BITS, IPT, false>;
         uint32_t* kout = (k + 1 == plan.passes && !keys_out) ? nullptr : keys[cur ^ 1];
-        kern<<<gs, kThreads, smem, s>>>(keys[cur], vals[cur], kout, vals[cur ^ 1], n, d_n,
-                                                 plan.shift[k], sc.ghist + k * BINS, sc.counters + k,
-                                                 sc.status + (int64_t)k * tiles_cap * BINS, sc.err,
-                                                 (k == 0 && sc.stall_test) ? 1 : 0);
+        kern<<<gs, kThreads, smem, s>>>(keys[cur], vals[cur], kout, vals[cur ^ 1], n, d_n, cap,
+                                        plan.shift[k], sc.ghist + k * BINS, sc.counters + k,
+                                        sc.status + k * sl.pass_words, sc.err,
+                                        (k == 0 && sc.stall_test) ? 1 : 0);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         cur ^= 1;
     }
     *result_buf = cur;
     return cudaSuccess;
+}
+
+template <int BITS>
+cudaError_t sort_b(uint32_t* keys[2], uint32_t* vals[2], int64_t n, const uint32_t* d_n, int64_t cap, int64_t expect,
+                   const SortPlan& plan, const SortScratch& sc, cudaStream_t s, int* result_buf,
+                   const char* const names[2], bool identity_vals, bool keys_out) {
+    if (sweep_ipt(expect) == 4)
+        return sort_t<BITS, 4>(keys, vals, n, d_n, cap, plan, sc, s, result_buf, names, identity_vals, keys_out);
+    return sort_t<BITS, 16>(keys, vals, n, d_n, cap, plan, sc, s, result_buf, names, identity_vals, keys_out);
 }
 
 }  // namespace
@@ -466,24 +594,25 @@ SortPlan make_sort_plan(int bits) {
     return p;
 }
 
-int64_t sort_status_words(const SortPlan& plan, int64_t cap) {
+int64_t sort_status_words(const SortPlan& plan, int64_t cap, int64_t expect) {
     if (plan.passes == 0) return 0;
-    return (int64_t)plan.passes * ((cap + kSortTile - 1) / kSortTile) * (1 << plan.digit_bits[0]);
+    const StatusLayout l = status_layout<0>(cap, kThreads * sweep_ipt(expect));
+    return plan.passes * (l.pass_words << plan.digit_bits[0]);
 }
 
 cudaError_t radix_sort(uint32_t* keys[2], uint32_t* vals[2], int64_t n, const uint32_t* d_n, int64_t cap,
-                       const SortPlan& plan, const SortScratch& sc, cudaStream_t s, int* result_buf,
+                       int64_t expect, const SortPlan& plan, const SortScratch& sc, cudaStream_t s, int* result_buf,
                        const char* const names[2], bool identity_vals, bool keys_out) {
     *result_buf = 0;
     if (plan.passes == 0 || cap == 0) return cudaSuccess;
     if (plan.passes > kMaxSortPasses) return cudaErrorInvalidValue;
     switch (plan.digit_bits[0]) {
-        case 4: return sort_t<4>(keys, vals, n, d_n, cap, plan, sc, s, result_buf, names, identity_vals, keys_out);
-        case 5: return sort_t<5>(keys, vals, n, d_n, cap, plan, sc, s, result_buf, names, identity_vals, keys_out);
-        case 6: return sort_t<6>(keys, vals, n, d_n, cap, plan, sc, s, result_buf, names, identity_vals, keys_out);
-        case 7: return sort_t<7>(keys, vals, n, d_n, cap, plan, sc, s, result_buf, names, identity_vals, keys_out);
-        case 8: return sort_t<8>(keys, vals, n, d_n, cap, plan, sc, s, result_buf, names, identity_vals, keys_out);
-        case 9: return sort_t<9>(keys, vals, n, d_n, cap, plan, sc, s, result_buf, names, identity_vals, keys_out);
+        case 4: return sort_b<4>(keys, vals, n, d_n, cap, expect, plan, sc, s, result_buf, names, identity_vals, keys_out);
+        case 5: return sort_b<5>(keys, vals, n, d_n, cap, expect, plan, sc, s, result_buf, names, identity_vals, keys_out);
+        case 6: return sort_b<6>(keys, vals, n, d_n, cap, expect, plan, sc, s, result_buf, names, identity_vals, keys_out);
+        case 7: return sort_b<7>(keys, vals, n, d_n, cap, expect, plan, sc, s, result_buf, names, identity_vals, keys_out);
+        case 8: return sort_b<8>(keys, vals, n, d_n, cap, expect, plan, sc, s, result_buf, names, identity_vals, keys_out);
+        case 9: return sort_b<9>(keys, vals, n, d_n, cap, expect, plan, sc, s, result_buf, names, identity_vals, keys_out);
         default: return cudaErrorInvalidValue;
     }
 }
