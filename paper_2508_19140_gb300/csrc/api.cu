@@ -63,6 +63,7 @@ struct Plan {
     int64_t copy_cap, blk_cap;
     int64_t expectA, expectC;  // elements the two sorts are expected to have (their launch shapes)
     SortPlan planA, planC;
+    RectCarry carry;      // rects carried through the depth sort
     int partial_floats;
     int arrangement;
     bool save_tiled;  // the forward writes the tile-ordered record copy
@@ -218,6 +219,8 @@ rast_status_t make_plan(const rast_view_t* views, int32_t n_views, const rast_op
     // reads each image's packed rects as a contiguous slice rather than
     // gathering over the whole batch.
     uint64_t key_max = max_cull;
+    RectCarry& rc = pl.carry;
+    int64_t img_points = npt;  // most points of one image (index bits of the carried rects)
     {
         const int db = bit_length(max_cull);
         int nimg = 0;
@@ -233,10 +236,38 @@ rast_status_t make_plan(const rast_view_t* views, int32_t n_views, const rast_op
                 vt.v[k].key_cull += hi;
             }
             key_max = ((uint64_t)(nimg - 1) << db) | max_cull;
+            rc.img_bits = ib;
+            rc.img_shift = db;
+            img_points = 0;
+            img = -1;
+            for (int k = 0; k < n_views; ++k) {
+                if (!(cont && cont[k] && k > 0)) rc.img_off[++img] = (uint32_t)vt.v[k].pt_off;
+                const int64_t in_img = vt.v[k].pt_off + vt.v[k].n - rc.img_off[img];
+                if (in_img > img_points) img_points = in_img;
+            }
         }
     }
     pl.planA = make_sort_plan(bit_length(key_max));
     pl.planC = make_sort_plan(bit_length((uint64_t)(ntile > 0 ? ntile - 1 : 0)));
+    // The rects travel with the depth sort when their code fits beside key and
+    // index (any usual frame: 27-bit keys, up to 32 M points, 1920x1080 at 8x8
+    // tiles); else the duplication gathers them in depth order.
+    {
+        int tx = 0, ty = 0;
+        for (int k = 0; k < n_views; ++k) {
+            if (vt.v[k].tiles_x > tx) tx = vt.v[k].tiles_x;
+            if (vt.v[k].tiles_y > ty) ty = vt.v[k].tiles_y;
+        }
+        rc.tx_bits = bit_length((uint64_t)tx);
+        rc.ty_bits = bit_length((uint64_t)ty);
+        rc.span_bits = o->mode == RAST_SPLAT_BILINEAR ? 1 : 2;
+        rc.bits = rc.tx_bits + rc.ty_bits + 2 * rc.span_bits;
+        rc.first_bits = pl.planA.digit_bits[0];
+        rc.rem_bits = pl.planA.bits - rc.first_bits;
+        rc.idx_bits = bit_length((uint64_t)(img_points > 1 ? img_points - 1 : 1));
+        rc.on = arrangement == kTiled && pl.planA.passes >= 2 && rc.bits <= kRectCarryMax &&
+                rc.bits <= (32 - rc.rem_bits) + (32 - rc.idx_bits);
+    }
     pl.partial_floats = partial_stride(o->mode == RAST_SPLAT_BILINEAR ? C + 1 : C + 7);
 
     const int64_t N = npt, D = pl.copy_cap;
@@ -431,21 +462,23 @@ cudaError_t run_fwd(const Plan& pl, const Bufs& b, cudaStream_t s) {
         RAST_TRY(cudaGetLastError());
     }
     // The depth sort's first pass generates the point indices itself.
-    RAST_TRY(launch_project(vt, b, pl.planA.passes == 0, s));
+    RAST_TRY(launch_project(vt, b, pl.planA.passes == 0, pl.carry, s));
     int ra = 0, rc = 0;
     {
         uint32_t* k[2] = {b.keyA[0], b.keyA[1]};
         uint32_t* v[2] = {b.valA[0], b.valA[1]};
         const SortScratch sc{b.sort_ghist, b.sort_counters, b.sort_status, &b.hdr->error,
                              (vt.flags & RAST_FLAG_TEST_SORT_STALL) != 0};
-        // Only the depth order of the point indices is used after this sort.
+        const CarryIo io{pl.carry, vt.mode == 0 ? b.rect4 : b.valA[0], vt.mode == 1, b.rect, b.rectS};
+        // Only the depth order of the point indices (and the points' rects in
+        // that order) is used after this sort.
         RAST_TRY(radix_sort(k, v, vt.n_total, nullptr, vt.n_total, pl.expectA, pl.planA, sc, s, &ra, kDepthSortNames,
-                            true, false));
+                            true, false, pl.carry.on ? &io : nullptr));
     }
     const uint32_t* depth_sorted = b.valA[ra];
     // A depth sort whose look-back wait ran out leaves a partial order: the
     // duplication then sees the error bit and writes no copies.
-    RAST_TRY(launch_duplicate(vt, b, depth_sorted, s));
+    RAST_TRY(launch_duplicate(vt, b, depth_sorted, pl.carry.on != 0, s));
     {
         uint32_t* k[2] = {b.keyC[0], b.keyC[1]};
         uint32_t* v[2] = {b.valC[0], b.valC[1]};
@@ -483,7 +516,7 @@ cudaError_t run_fwd_key64(const Plan& pl, const Bufs& b, cudaStream_t s) {
                                       vt.pix_total, pl.save_tiled ? 1u : 0u);
         RAST_TRY(cudaGetLastError());
     }
-    RAST_TRY(launch_project(vt, b, false, s));
+    RAST_TRY(launch_project(vt, b, false, RectCarry{}, s));
     RAST_TRY(launch_untiled_copies(vt, b, b.keyA[0], b.keyC[0], b.pixC, b.ptC, s));
     const SortScratch sc{b.sort_ghist, b.sort_counters, b.sort_status, &b.hdr->error,
                          (vt.flags & RAST_FLAG_TEST_SORT_STALL) != 0};

@@ -65,8 +65,8 @@ __device__ __forceinline__ void load_point(const ViewTable& vt, const ViewDev& V
 }
 
 template <int MODE>
-__device__ __forceinline__ void project_point(const ViewTable& vt, const Bufs& b, bool write_vals, int64_t gi,
-                                              const ViewDev& V, int64_t i, const PointIn& in) {
+__device__ __forceinline__ void project_point(const ViewTable& vt, const Bufs& b, bool write_vals,
+                                              const RectCarry& rc, int64_t gi, const ViewDev& V, int64_t i, const PointIn& in) {
     const float x = in.x, y = in.y, z = in.z;
     float xc = __fmul_rn(V.R[0], x);
     xc = __fadd_rn(xc, __fmul_rn(V.R[1], y));
@@ -198,6 +198,10 @@ __device__ __forceinline__ void project_point(const ViewTable& vt, const Bufs& b
     }
     b.keyA[0][gi] = key;
     if (write_vals) b.valA[0][gi] = (uint32_t)gi;
+    if (MODE == 1 && rc.on)
+        b.valA[0][gi] = vis ? rect_code(rc, rect.x & 0xffffu, rect.x >> 16, (rect.y & 0xffffu) - (rect.x & 0xffffu),
+                                        (rect.y >> 16) - (rect.x >> 16))
+                            : rect_code_empty(rc);
     if (MODE == 0)
         b.rect4[gi] = vis ? rect4_pack((int)(rect.x & 0xffffu), (int)(rect.x >> 16), (int)(rect.y & 0xffffu),
                                        (int)(rect.y >> 16))
@@ -214,7 +218,8 @@ __device__ __forceinline__ void project_point(const ViewTable& vt, const Bufs& b
 constexpr int kPointsPerThread = 2;
 
 template <int MODE>
-__global__ void __launch_bounds__(256) k_project(const ViewTable vt, const Bufs b, bool write_vals) {
+__global__ void __launch_bounds__(256) k_project(const ViewTable vt, const Bufs b, bool write_vals,
+                                                 const RectCarry rc) {
     constexpr int K = kPointsPerThread;
     const int64_t g0 = (int64_t)blockIdx.x * (256 * K) + threadIdx.x;
     PointIn in[K];
@@ -234,19 +239,19 @@ __global__ void __launch_bounds__(256) k_project(const ViewTable vt, const Bufs 
         const int64_t gi = g0 + k * 256;
         if (gi < vt.n_total) {
             const ViewDev& V = vt.v[vi[k]];
-            project_point<MODE>(vt, b, write_vals, gi, V, gi - V.pt_off, in[k]);
+            project_point<MODE>(vt, b, write_vals, rc, gi, V, gi - V.pt_off, in[k]);
         }
     }
 }
 
 }  // namespace
 
-cudaError_t launch_project(const ViewTable& vt, const Bufs& b, bool write_vals, cudaStream_t s) {
+cudaError_t launch_project(const ViewTable& vt, const Bufs& b, bool write_vals, const RectCarry& rc, cudaStream_t s) {
     if (vt.n_total == 0) return cudaSuccess;
     const unsigned grid = (unsigned)((vt.n_total + 256 * kPointsPerThread - 1) / (256 * kPointsPerThread));
     ProfScope ps("project", s);
-    if (vt.mode == 0) k_project<0><<<grid, 256, 0, s>>>(vt, b, write_vals);
-    else k_project<1><<<grid, 256, 0, s>>>(vt, b, write_vals);
+    if (vt.mode == 0) k_project<0><<<grid, 256, 0, s>>>(vt, b, write_vals, rc);
+    else k_project<1><<<grid, 256, 0, s>>>(vt, b, write_vals, rc);
     return cudaGetLastError();
 }
 

@@ -259,6 +259,7 @@ constexpr int kMaxSortPasses = 4;
 
 struct SortPlan {
     int passes;
+    int bits;  // of the keys
     int digit_bits[8];
     int shift[8];
 };
@@ -266,6 +267,33 @@ SortPlan make_sort_plan(int bits);
 // Look-back words one sort with this plan needs for `cap` elements, launched
 // for about `expect` of them.
 int64_t sort_status_words(const SortPlan& plan, int64_t cap, int64_t expect);
+
+// Tile rects carried through the depth sort. A point's rect packs into `bits`
+// bits: tx0 | ty0 | (tx1 - tx0) | (ty1 - ty0), the spans in span_bits each (1
+// for bilinear points; 2 for Gaussians, where a column span of 3 stands for a
+// rect too large for the code); all ones = empty (tx_bits hold tiles_x, so no
+// column is all ones). The first pass drops the digit it has sorted by and puts
+// the code into the freed key bits and into those above the point index, which
+// is counted from the first point of the point's image; the last pass unpacks.
+struct RectCarry {
+    int32_t on;        // 0: the code does not fit, the duplication gathers the rects
+    int32_t tx_bits, ty_bits, span_bits, bits;
+    int32_t first_bits;  // bits of the first digit
+    int32_t rem_bits;    // key bits left after it
+    int32_t idx_bits;    // bits of a point index within its image
+    int32_t img_bits, img_shift;  // image index: the key's top bits (0: one image)
+    uint32_t img_off[kMaxViews];  // first point of every image
+};
+constexpr int kRectCarryMax = 20;  // code bits: a 4096-key tile's positions share a word with it
+
+__host__ __device__ __forceinline__ uint32_t rect_code_empty(const RectCarry& rc) { return (1u << rc.bits) - 1u; }
+
+// Code of a rect (inclusive tile corners).
+__device__ __forceinline__ uint32_t rect_code(const RectCarry& rc, uint32_t tx0, uint32_t ty0, uint32_t w, uint32_t h) {
+    const uint32_t top = (1u << rc.span_bits) - 1u;
+    if (rc.span_bits > 1 && (w >= top || h >= top)) w = top, h = 0;  // escape
+    return tx0 | (ty0 << rc.tx_bits) | (w << (rc.tx_bits + rc.ty_bits)) | (h << (rc.tx_bits + rc.ty_bits + rc.span_bits));
+}
 
 struct SortScratch {
     uint32_t* ghist;     // [kMaxSortPasses][512]
@@ -275,9 +303,19 @@ struct SortScratch {
     bool stall_test = false;  // RAST_FLAG_TEST_SORT_STALL: the first pass's first tile never publishes
 };
 
+struct CarryIo {
+    RectCarry rc;
+    const uint32_t* in;   // per point: rect4 (bilinear) or the rect's code (Gaussian)
+    bool coded;           // `in` holds codes
+    const uint2* full;    // Gaussian: rects of the points whose code is the escape
+    void* out;            // rects in sorted order: rect4 (bilinear) or uint2
+};
+
 // write_vals: also write the identity point values into valA[0] (needed only
-// when the depth sort makes no pass).
-cudaError_t launch_project(const ViewTable& vt, const Bufs& b, bool write_vals, cudaStream_t s);
+// when the depth sort makes no pass). rc: with rects carried through the depth
+// sort, Gaussian points write their rect's code into valA[0] (bilinear ones are
+// coded from rect4 by the sort).
+cudaError_t launch_project(const ViewTable& vt, const Bufs& b, bool write_vals, const RectCarry& rc, cudaStream_t s);
 // Stable LSD radix sort of (key, val) pairs in keys[0]/vals[0] using keys[1]/vals[1]
 // as scratch; count from d_n (device) if non-null else n (at most cap); expect:
 // the count the launch shapes are chosen for. Sets *result_buf to the index (0/1) of the buffer that holds the result.
@@ -285,10 +323,14 @@ cudaError_t launch_project(const ViewTable& vt, const Bufs& b, bool write_vals, 
 // identity_vals: the input values are their own positions (0, 1, 2, ...);
 // vals[0] is then not read. keys_out = false: only the values are wanted, the
 // last pass does not write keys (keys[*result_buf] is left stale).
+// carry: the values are point indices (identity_vals) and every point's rect
+// goes with them (at least two passes).
 cudaError_t radix_sort(uint32_t* keys[2], uint32_t* vals[2], int64_t n, const uint32_t* d_n, int64_t cap,
                        int64_t expect, const SortPlan& plan, const SortScratch& sc, cudaStream_t s, int* result_buf,
-                       const char* const names[2], bool identity_vals = false, bool keys_out = true);
-cudaError_t launch_duplicate(const ViewTable& vt, const Bufs& b, const uint32_t* sorted_pts,
+                       const char* const names[2], bool identity_vals = false, bool keys_out = true,
+                       const CarryIo* carry = nullptr);
+// carried: the depth sort has written rectS / rect4S.
+cudaError_t launch_duplicate(const ViewTable& vt, const Bufs& b, const uint32_t* sorted_pts, bool carried,
                              cudaStream_t s);
 cudaError_t launch_ranges(const ViewTable& vt, const Bufs& b, const uint32_t* sorted_tiles,
                           cudaStream_t s);

@@ -236,8 +236,30 @@ constexpr size_t sweep_smem() {
     return 128 + sizeof(uint32_t) * (3 * kThreads * IPT + (2 * kWarps + 2) * (1 << BITS));
 }
 
-// IDV: the input values are their positions (not read from memory).
-//
+// What a sweep moves with its keys.
+enum SweepKind {
+    kPairs = 0,     // values as they are
+    kIdentity = 1,  // the input values are their positions (not read from memory)
+    kCarryIn = 2,   // first depth pass: the values are positions, their rects are read and packed with them
+    kCarryOut = 3   // last depth pass: writes the point indices and the rects
+};
+
+// A key and a value as the first pass of a sort that carries rects writes
+// them: the key without its first digit below the code's low bits, the index
+// within the image below the code's high bits.
+__device__ __forceinline__ uint2 carry_pack(const RectCarry& rc, uint32_t key, uint32_t gi, uint32_t code) {
+    const uint32_t off = rc.img_bits ? rc.img_off[key >> rc.img_shift] : 0u;
+    return make_uint2((key >> rc.first_bits) | (code << rc.rem_bits),
+                      (gi - off) | ((code >> (32 - rc.rem_bits)) << rc.idx_bits));
+}
+
+__device__ __forceinline__ void carry_unpack(const RectCarry& rc, uint32_t k, uint32_t v, uint32_t& gi, uint32_t& code) {
+    const uint32_t rem = k & ((1u << rc.rem_bits) - 1u);
+    const uint32_t off = rc.img_bits ? rc.img_off[rem >> (rc.rem_bits - rc.img_bits)] : 0u;
+    gi = (v & ((1u << rc.idx_bits) - 1u)) + off;
+    code = ((k >> rc.rem_bits) | ((v >> rc.idx_bits) << (32 - rc.rem_bits))) & ((1u << rc.bits) - 1u);
+}
+
 // Tiles arrive by TMA bulk copies, one for the keys and one for the values,
 // into three shared buffers that change roles from tile to tile: the keys are
 // read into registers and sorted in place, the values go from their buffer to
@@ -254,12 +276,13 @@ constexpr size_t sweep_smem() {
 // with the next tile on its way beat four without: 147 us. The whole pass went
 // 217 -> 147 us (32 M keys, 7-bit digits; 3.6 TB/s moved), 36.6 -> 27 us (4 M
 // keys), 433 -> 308 us (62 M keys, 8-bit), 630 -> 535 us (77 M keys, 9-bit).
-template <int BITS, int IPT, bool IDV>
+template <int BITS, int IPT, int KIND>
 __global__ void __launch_bounds__(kThreads, IPT == 16 ? 3 : 4) k_sweep(
     const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint32_t* __restrict__ kout,
     uint32_t* __restrict__ vout, int64_t n_host, const uint32_t* d_n, int64_t cap, int shift,
-    const uint32_t* __restrict__ ghist_pass, uint32_t* __restrict__ counter, uint32_t* __restrict__ status,
-    uint32_t* __restrict__ err, int stall_test) {
+    uint32_t mask, const uint32_t* __restrict__ ghist_pass, uint32_t* __restrict__ counter,
+    uint32_t* __restrict__ status, uint32_t* __restrict__ err, int stall_test, const CarryIo carry) {
+    constexpr bool IDV = KIND == kIdentity;
     constexpr int BINS = 1 << BITS;
     constexpr int VPT = BINS > kThreads ? BINS / kThreads : 1;  // consecutive bins per thread
     constexpr int TILE = kThreads * IPT;
@@ -350,7 +373,7 @@ __global__ void __launch_bounds__(kThreads, IPT == 16 ? 3 : 4) k_sweep(
         }
         __syncwarp();
 #pragma unroll
-        for (int r = 0; r < IPT; ++r) atomicAdd(&tab[(k[r] >> shift) & (BINS - 1)].y, 1u);
+        for (int r = 0; r < IPT; ++r) atomicAdd(&tab[(k[r] >> shift) & mask].y, 1u);
         if (__syncthreads_or(failed)) {  // a copy never arrived: report it, let the other land, stop
             if (tid == 0) atomicOr(err, kErrTimeout);
             mbar_wait(&s_mbar[0], phase);
@@ -375,7 +398,7 @@ __global__ void __launch_bounds__(kThreads, IPT == 16 ? 3 : 4) k_sweep(
                     c[q][w] = s_tab[w * BINS + bin].y;
                     sum += c[q][w];
                 }
-                tot[q] = sum - (bin == BINS - 1 ? (uint32_t)(TILE - cnt) : 0u);
+                tot[q] = sum - (bin == (int)mask ? (uint32_t)(TILE - cnt) : 0u);
                 if (publish) {
                     st_relaxed(status + tile * BINS + bin, kFlag | tot[q]);
                     atomicAdd(&groups[(tile / kGroup) * BINS + bin].y, kArrival | tot[q]);
@@ -413,7 +436,7 @@ __global__ void __launch_bounds__(kThreads, IPT == 16 ? 3 : 4) k_sweep(
         // Stable rank: rounds in input order, lanes in order within a round.
 #pragma unroll
         for (int r = 0; r < IPT; ++r) {
-            const uint32_t d = (k[r] >> shift) & (BINS - 1);
+            const uint32_t d = (k[r] >> shift) & mask;
             uint32_t peers, pre;  // lanes holding the same digit; the digit's next position
             if (r & 1) {
                 peers = 0xffffffffu;
@@ -436,7 +459,20 @@ __global__ void __launch_bounds__(kThreads, IPT == 16 ? 3 : 4) k_sweep(
             if (below == 0) tab[d] = make_uint2(0u, pre + __popc(peers));
             __syncwarp();
             s_k[pre + below] = k[r];
-            s_s[pre + below] = IDV ? (uint32_t)base + (uint32_t)(w0 + r * 32) : s_v[w0 + r * 32];
+            uint32_t v;
+            if constexpr (KIND == kIdentity) {
+                v = (uint32_t)base + (uint32_t)(w0 + r * 32);
+            } else {
+                v = s_v[w0 + r * 32];
+                if constexpr (KIND == kCarryIn) {
+                    // the rect's code and the key's position in the tile
+                    if (!carry.coded)
+                        v = v == kRect4Empty ? rect_code_empty(carry.rc)
+                                             : rect_code(carry.rc, v & 0xffffu, (v >> 16) & 0x3fffu, (v >> 30) & 1u, v >> 31);
+                    v = (v << 12) | (uint32_t)(w0 + r * 32);
+                }
+            }
+            s_s[pre + below] = v;
         }
 #pragma unroll
         for (int q = 0; q < VPT; ++q) {
@@ -453,6 +489,35 @@ __global__ void __launch_bounds__(kThreads, IPT == 16 ? 3 : 4) k_sweep(
         tile = s_tile;
         if (tid == 0 && tile < ntiles) fetch(s_v, kin, tile, &s_mbar[0]);
 
+        auto put = [&](uint32_t key, uint32_t val, uint32_t dst) {
+            if constexpr (KIND == kCarryIn) {
+                const uint2 e = carry_pack(carry.rc, key, (uint32_t)base + (val & 4095u), val >> 12);
+                kout[dst] = e.x;
+                vout[dst] = e.y;
+            } else if constexpr (KIND == kCarryOut) {
+                const RectCarry& rc = carry.rc;
+                uint32_t gi, code;
+                carry_unpack(rc, key, val, gi, code);
+                vout[dst] = gi;
+                const uint32_t tx0 = code & ((1u << rc.tx_bits) - 1u), ty0 = (code >> rc.tx_bits) & ((1u << rc.ty_bits) - 1u);
+                const uint32_t span = code >> (rc.tx_bits + rc.ty_bits);
+                if (!carry.coded) {
+                    static_cast<uint32_t*>(carry.out)[dst] =
+                        code == rect_code_empty(rc) ? kRect4Empty : tx0 | (ty0 << 16) | (span << 30);
+                } else {
+                    uint2 q = make_uint2(1u, 0u);
+                    if (code != rect_code_empty(rc)) {
+                        const uint32_t w = span & 3u, h = span >> 2;
+                        q = w == 3u ? ((int64_t)gi < n ? carry.full[gi] : q)
+                                    : make_uint2(tx0 | (ty0 << 16), (tx0 + w) | ((ty0 + h) << 16));
+                    }
+                    static_cast<uint2*>(carry.out)[dst] = q;
+                }
+            } else {
+                if (kout) kout[dst] = key;
+                vout[dst] = val;
+            }
+        };
         if (cnt == TILE) {
             constexpr int U = 4;
 #pragma unroll 1
@@ -465,19 +530,15 @@ __global__ void __launch_bounds__(kThreads, IPT == 16 ? 3 : 4) k_sweep(
                 }
 #pragma unroll
                 for (int u = 0; u < U; ++u)
-                    dst[u] = s_ofs[(key[u] >> shift) & (BINS - 1)] + (uint32_t)(j0 + u * kThreads);
+                    dst[u] = s_ofs[(key[u] >> shift) & mask] + (uint32_t)(j0 + u * kThreads);
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    if (kout) kout[dst[u]] = key[u];
-                    vout[dst[u]] = val[u];
-                }
+                for (int u = 0; u < U; ++u) put(key[u], val[u], dst[u]);
             }
         } else {
             for (int j = tid; j < cnt; j += kThreads) {
                 const uint32_t key = s_k[j];
-                const uint32_t dst = s_ofs[(key >> shift) & (BINS - 1)] + (uint32_t)j;
-                if (kout) kout[dst] = key;
-                vout[dst] = s_s[j];
+                const uint32_t dst = s_ofs[(key >> shift) & mask] + (uint32_t)j;
+                put(key, s_s[j], dst);
             }
         }
         fence_proxy_async();
@@ -500,7 +561,7 @@ int sweep_ipt(int64_t expect) { return expect <= 256 * 1024 ? 4 : 16; }
 template <int BITS, int IPT>
 cudaError_t sort_t(uint32_t* keys[2], uint32_t* vals[2], int64_t n, const uint32_t* d_n, int64_t cap,
                    const SortPlan& plan, const SortScratch& sc, cudaStream_t s, int* result_buf,
-                   const char* const names[2], bool identity_vals, bool keys_out) {
+                   const char* const names[2], bool identity_vals, bool keys_out, const CarryIo* carry) {
     constexpr int BINS = 1 << BITS;
     constexpr int TILE = kThreads * IPT;
     // Launch attributes and the resident CTAs per SM of the sweep, once per
@@ -511,14 +572,14 @@ cudaError_t sort_t(uint32_t* keys[2], uint32_t* vals[2], int64_t n, const uint32
     int per_sm = 1;
     cudaError_t e = per_device(setup, &per_sm, [](int, int* v) {
         *v = 1;
-        cudaError_t r = cudaFuncSetAttribute(k_sweep<BITS, IPT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (r == cudaSuccess)
-            r = cudaFuncSetAttribute(k_sweep<BITS, IPT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem);
+        cudaError_t r = cudaSuccess;
+        for (auto kern : {k_sweep<BITS, IPT, kPairs>, k_sweep<BITS, IPT, kIdentity>, k_sweep<BITS, IPT, kCarryIn>,
+                          k_sweep<BITS, IPT, kCarryOut>})
+            if (r == cudaSuccess)
+                r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (r != cudaSuccess) return r;
         int occ = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_sweep<BITS, IPT, false>, kThreads, smem) ==
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_sweep<BITS, IPT, kPairs>, kThreads, smem) ==
                 cudaSuccess && occ >= 1)
             *v = occ;
         return cudaSuccess;
@@ -544,12 +605,26 @@ cudaError_t sort_t(uint32_t* keys[2], uint32_t* vals[2], int64_t n, const uint32
     int cur = 0;
     for (int k = 0; k < plan.passes; ++k) {
         ProfScope ps(names[1], s);
-        auto kern = (k == 0 && identity_vals) ? k_sweep<BITS, IPT, true> : k_sweep<BITS, IPT, false>;
-        uint32_t* kout = (k + 1 == plan.passes && !keys_out) ? nullptr : keys[cur ^ 1];
-        kern<<<gs, kThreads, smem, s>>>(keys[cur], vals[cur], kout, vals[cur ^ 1], n, d_n, cap,
-                                        plan.shift[k], sc.ghist + k * BINS, sc.counters + k,
-                                        sc.status + k * sl.pass_words, sc.err,
-                                        (k == 0 && sc.stall_test) ? 1 : 0);
+        const bool last = k + 1 == plan.passes;
+        auto kern = k_sweep<BITS, IPT, kPairs>;
+        const uint32_t* vin = vals[cur];
+        int shift = plan.shift[k];
+        uint32_t mask = BINS - 1;
+        if (carry) {
+            // after the first pass the key's first digit is gone, and other bits stand above the key
+            const int left = plan.bits - plan.shift[k];
+            if (left < BITS) mask = (1u << left) - 1u;
+            if (k > 0) shift -= plan.digit_bits[0];
+            if (k == 0) vin = carry->in;
+            if (k == 0) kern = k_sweep<BITS, IPT, kCarryIn>;
+            else if (last) kern = k_sweep<BITS, IPT, kCarryOut>;
+        } else if (k == 0 && identity_vals) {
+            kern = k_sweep<BITS, IPT, kIdentity>;
+        }
+        uint32_t* kout = (last && !keys_out) ? nullptr : keys[cur ^ 1];
+        kern<<<gs, kThreads, smem, s>>>(keys[cur], vin, kout, vals[cur ^ 1], n, d_n, cap, shift, mask,
+                                        sc.ghist + k * BINS, sc.counters + k, sc.status + k * sl.pass_words, sc.err,
+                                        (k == 0 && sc.stall_test) ? 1 : 0, carry ? *carry : CarryIo{});
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         cur ^= 1;
@@ -561,10 +636,10 @@ cudaError_t sort_t(uint32_t* keys[2], uint32_t* vals[2], int64_t n, const uint32
 template <int BITS>
 cudaError_t sort_b(uint32_t* keys[2], uint32_t* vals[2], int64_t n, const uint32_t* d_n, int64_t cap, int64_t expect,
                    const SortPlan& plan, const SortScratch& sc, cudaStream_t s, int* result_buf,
-                   const char* const names[2], bool identity_vals, bool keys_out) {
+                   const char* const names[2], bool identity_vals, bool keys_out, const CarryIo* carry) {
     if (sweep_ipt(expect) == 4)
-        return sort_t<BITS, 4>(keys, vals, n, d_n, cap, plan, sc, s, result_buf, names, identity_vals, keys_out);
-    return sort_t<BITS, 16>(keys, vals, n, d_n, cap, plan, sc, s, result_buf, names, identity_vals, keys_out);
+        return sort_t<BITS, 4>(keys, vals, n, d_n, cap, plan, sc, s, result_buf, names, identity_vals, keys_out, carry);
+    return sort_t<BITS, 16>(keys, vals, n, d_n, cap, plan, sc, s, result_buf, names, identity_vals, keys_out, carry);
 }
 
 }  // namespace
@@ -591,6 +666,7 @@ SortPlan make_sort_plan(int bits) {
         shift += per;
     }
     p.passes = passes;
+    p.bits = bits;
     return p;
 }
 
@@ -602,17 +678,17 @@ int64_t sort_status_words(const SortPlan& plan, int64_t cap, int64_t expect) {
 
 cudaError_t radix_sort(uint32_t* keys[2], uint32_t* vals[2], int64_t n, const uint32_t* d_n, int64_t cap,
                        int64_t expect, const SortPlan& plan, const SortScratch& sc, cudaStream_t s, int* result_buf,
-                       const char* const names[2], bool identity_vals, bool keys_out) {
+                       const char* const names[2], bool identity_vals, bool keys_out, const CarryIo* carry) {
     *result_buf = 0;
     if (plan.passes == 0 || cap == 0) return cudaSuccess;
     if (plan.passes > kMaxSortPasses) return cudaErrorInvalidValue;
     switch (plan.digit_bits[0]) {
-        case 4: return sort_b<4>(keys, vals, n, d_n, cap, expect, plan, sc, s, result_buf, names, identity_vals, keys_out);
-        case 5: return sort_b<5>(keys, vals, n, d_n, cap, expect, plan, sc, s, result_buf, names, identity_vals, keys_out);
-        case 6: return sort_b<6>(keys, vals, n, d_n, cap, expect, plan, sc, s, result_buf, names, identity_vals, keys_out);
-        case 7: return sort_b<7>(keys, vals, n, d_n, cap, expect, plan, sc, s, result_buf, names, identity_vals, keys_out);
-        case 8: return sort_b<8>(keys, vals, n, d_n, cap, expect, plan, sc, s, result_buf, names, identity_vals, keys_out);
-        case 9: return sort_b<9>(keys, vals, n, d_n, cap, expect, plan, sc, s, result_buf, names, identity_vals, keys_out);
+        case 4: return sort_b<4>(keys, vals, n, d_n, cap, expect, plan, sc, s, result_buf, names, identity_vals, keys_out, carry);
+        case 5: return sort_b<5>(keys, vals, n, d_n, cap, expect, plan, sc, s, result_buf, names, identity_vals, keys_out, carry);
+        case 6: return sort_b<6>(keys, vals, n, d_n, cap, expect, plan, sc, s, result_buf, names, identity_vals, keys_out, carry);
+        case 7: return sort_b<7>(keys, vals, n, d_n, cap, expect, plan, sc, s, result_buf, names, identity_vals, keys_out, carry);
+        case 8: return sort_b<8>(keys, vals, n, d_n, cap, expect, plan, sc, s, result_buf, names, identity_vals, keys_out, carry);
+        case 9: return sort_b<9>(keys, vals, n, d_n, cap, expect, plan, sc, s, result_buf, names, identity_vals, keys_out, carry);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -46,16 +46,23 @@ def _check(views, tile=16):
     # (image, depth bits, index): culled points behind every visible one of their image
     depth = np.lexsort((np.arange(n), np.where(p4 == 0xFFFFFFFF, cull, zb), image))
     assert np.array_equal(r.arr("depth_sorted", np.uint32, n), depth.astype(np.uint32))
-    # copies in that order, row by row of each point's tile rect, then stably by tile
+    _check_copies(r, views, tile, depth, image, (p4 & 0xFFFF, (p4 >> 16) & 0x3FFF, (p4 >> 30) & 1, p4 >> 31),
+                  p4 != 0xFFFFFFFF)
+
+
+def _check_copies(r, views, tile, depth, image, rect, visible):
+    """The copies in depth order, row by row of each point's tile rect (tx0, ty0, and
+    the spans), then stably by tile."""
     offs, grids = np.cumsum([0] + [-(-v.camera.width // tile) * -(-v.camera.height // tile) for v in views]), \
         np.array([-(-v.camera.width // tile) for v in views])
-    q, im = p4[depth], image[depth]
+    tx0, ty0, w, h = (x[depth] for x in rect)
+    im, vis = image[depth], visible[depth]
     tiles, pts = [], []
-    for k in range(4):  # the rect's tiles (dx, dy): at most two by two
-        dx, dy = k & 1, k >> 1
-        ok = (q != 0xFFFFFFFF) & (((q >> 30) & 1) >= dx) & ((q >> 31) >= dy)
-        tiles.append(np.where(ok, offs[im] + (((q >> 16) & 0x3FFF) + dy) * grids[im] + (q & 0xFFFF) + dx, -1))
-        pts.append(depth)
+    for dy in range(int(h[vis].max(initial=0)) + 1):
+        for dx in range(int(w[vis].max(initial=0)) + 1):
+            ok = vis & (w >= dx) & (h >= dy)
+            tiles.append(np.where(ok, offs[im] + (ty0 + dy) * grids[im] + tx0 + dx, -1))
+            pts.append(depth)
     tiles, pts = np.stack(tiles, 1).ravel(), np.stack(pts, 1).ravel()
     keep = tiles >= 0
     order = np.argsort(tiles[keep], kind="stable")
@@ -79,3 +86,32 @@ def test_sorts_with_few_distinct_keys(n, depths):
 def test_sorts_of_several_images_and_wide_tile_ids():
     # 2^18 tiles of 8x8 (9-bit tile digits) beside a small image: image-major depth keys
     _check([_view(70001, 4096, 4096, "spread", 1), _view(3000, 64, 48, "spread", 2)], tile=8)
+
+
+@pytest.mark.parametrize("tile", [8, 16])
+def test_rects_of_several_images_follow_the_depth_sort(tile):
+    _check([_view(20011, 320, 200, "spread", 3), _view(7, 64, 48, "spread", 4), _view(300007, 100, 75, "culled", 5)],
+           tile=tile)
+
+
+# small Gaussians (spans of up to two tiles), ones whose spans leave the rect's code (three
+# tiles and more), and an image too large for the code (its rects are gathered in depth order)
+@pytest.mark.parametrize("width,height,scale,tile", [(320, 200, 0.004, 16), (320, 200, 0.15, 16),
+                                                     (4096, 4096, 2e-4, 8)])
+@pytest.mark.parametrize("n", [3001, 300001])
+def test_gaussian_rects_follow_the_depth_sort(n, width, height, scale, tile):
+    if n > 10000 and scale > 0.1:
+        n = 20001  # many copies a point
+    rng = np.random.default_rng(n + width)
+    v = _view(n, width, height, "spread", n)
+    v.scale = (v.xyz[:, 2] * scale * rng.uniform(0.2, 1.0, n)).astype(np.float32)
+    v.scale[v.scale < 0] = 0.01
+    r = Run([v], mode="gaussian", tile=tile, max_copies=400 if scale > 0.1 else 0)
+    assert r.status == 0
+    rect = r.arr("rect", np.uint32, 2 * n).reshape(n, 2).astype(np.int64)
+    tx0, ty0, tx1, ty1 = rect[:, 0] & 0xFFFF, rect[:, 0] >> 16, rect[:, 1] & 0xFFFF, rect[:, 1] >> 16
+    visible = tx0 <= tx1
+    zb = r.arr("zbits", np.uint32, n).astype(np.int64)
+    depth = np.lexsort((np.arange(n), np.where(visible, zb, int(_bits(v.camera.far)))))
+    assert np.array_equal(r.arr("depth_sorted", np.uint32, n), depth.astype(np.uint32))
+    _check_copies(r, [v], tile, depth, np.zeros(n, np.int64), (tx0, ty0, tx1 - tx0, ty1 - ty0), visible)
