@@ -283,7 +283,7 @@ rast_status_t make_plan(const rast_view_t* views, int32_t n_views, const rast_op
     pl.bytes[S_KEYC0] = pl.bytes[S_KEYC1] = pl.bytes[S_VALC0] = pl.bytes[S_VALC1] = (size_t)D * 4;
     pl.bytes[S_PARTIAL] = (size_t)D * pl.partial_floats * 4;
     pl.bytes[S_GROW] = o->mode == RAST_SPLAT_BILINEAR ? (size_t)N * grow_stride(C + 1) * 4 : 0;
-    pl.bytes[S_SGHIST] = (size_t)kMaxSortPasses * 512 * 4;
+    pl.bytes[S_SGHIST] = (size_t)2 * kSortHistWords * 4;
     pl.bytes[S_SCOUNT] = (size_t)kMaxSortPasses * 4;
     int64_t sort_words;
     {
@@ -369,8 +369,16 @@ Bufs make_bufs(const Plan& pl, void* ws) {
     return b;
 }
 
-__global__ void k_init_header(WsHeader* h, int32_t n_views, long long n_points, long long cap,
-                              long long n_tiles, long long n_pixels, uint32_t rec_tile_valid) {
+// Header of a forward pass; the digit counts of both sorts and the tile order's
+// bucket counts cleared.
+constexpr int kBucketWords = 66;
+__global__ void __launch_bounds__(1024) k_init(WsHeader* h, int32_t n_views, long long n_points, long long cap,
+                                               long long n_tiles, long long n_pixels, uint32_t rec_tile_valid,
+                                               uint32_t* hist, uint32_t* buckets) {
+    static_assert(2 * kSortHistWords % 1024 == 0, "every thread clears whole strides");
+    for (int i = threadIdx.x; i < 2 * kSortHistWords; i += 1024) hist[i] = 0;
+    if (threadIdx.x < kBucketWords) buckets[threadIdx.x] = 0;
+    if (threadIdx.x != 0) return;
     h->rec_tile_valid = rec_tile_valid;
     h->error = 0u;
     h->n_copies = 0u;
@@ -453,14 +461,17 @@ namespace {
 const char* const kDepthSortNames[2] = {"depth_sort.hist", "depth_sort.sweep"};
 const char* const kTileSortNames[2] = {"tile_sort.hist", "tile_sort.sweep"};
 
+cudaError_t launch_init(const Plan& pl, const Bufs& b, cudaStream_t s) {
+    const ViewTable& vt = pl.vt;
+    ProfScope ps("init", s);
+    k_init<<<1, 1024, 0, s>>>(b.hdr, vt.n_views, vt.n_total, pl.copy_cap, vt.tiles_total, vt.pix_total,
+                              pl.save_tiled ? 1u : 0u, b.sort_ghist, b.order + vt.tiles_total);
+    return cudaGetLastError();
+}
+
 cudaError_t run_fwd(const Plan& pl, const Bufs& b, cudaStream_t s) {
     const ViewTable& vt = pl.vt;
-    {
-        ProfScope ps("init_header", s);
-        k_init_header<<<1, 1, 0, s>>>(b.hdr, vt.n_views, vt.n_total, pl.copy_cap, vt.tiles_total,
-                                      vt.pix_total, pl.save_tiled ? 1u : 0u);
-        RAST_TRY(cudaGetLastError());
-    }
+    RAST_TRY(launch_init(pl, b, s));
     // The depth sort's first pass generates the point indices itself.
     RAST_TRY(launch_project(vt, b, pl.planA.passes == 0, pl.carry, s));
     int ra = 0, rc = 0;
@@ -482,10 +493,10 @@ cudaError_t run_fwd(const Plan& pl, const Bufs& b, cudaStream_t s) {
     {
         uint32_t* k[2] = {b.keyC[0], b.keyC[1]};
         uint32_t* v[2] = {b.valC[0], b.valC[1]};
-        const SortScratch sc{b.sort_ghist, b.sort_counters, b.sort_status, &b.hdr->error};
+        const SortScratch sc{b.sort_ghist + kSortHistWords, b.sort_counters, b.sort_status, &b.hdr->error};
         RAST_TRY(radix_sort(k, v, 0, &b.hdr->n_copies, pl.copy_cap, pl.expectC, pl.planC, sc, s, &rc, kTileSortNames));
     }
-    RAST_TRY(launch_ranges(vt, b, b.keyC[rc], s));
+    RAST_TRY(launch_ranges(vt, b, b.keyC[rc], pl.expectC, s));
     if (vt.tile == 1) return launch_blend_fwd_pixel(vt, b, b.valC[rc], s);  // untiled baseline
     RAST_TRY(launch_tile_order(vt, b, s));
     RAST_TRY(launch_blend_fwd(vt, b, b.valC[rc], s));
@@ -510,12 +521,7 @@ int key64_result_pair(const Plan& pl) {
 
 cudaError_t run_fwd_key64(const Plan& pl, const Bufs& b, cudaStream_t s) {
     const ViewTable& vt = pl.vt;
-    {
-        ProfScope ps("init_header", s);
-        k_init_header<<<1, 1, 0, s>>>(b.hdr, vt.n_views, vt.n_total, pl.copy_cap, vt.tiles_total,
-                                      vt.pix_total, pl.save_tiled ? 1u : 0u);
-        RAST_TRY(cudaGetLastError());
-    }
+    RAST_TRY(launch_init(pl, b, s));
     RAST_TRY(launch_project(vt, b, false, RectCarry{}, s));
     RAST_TRY(launch_untiled_copies(vt, b, b.keyA[0], b.keyC[0], b.pixC, b.ptC, s));
     const SortScratch sc{b.sort_ghist, b.sort_counters, b.sort_status, &b.hdr->error,
@@ -535,19 +541,19 @@ cudaError_t run_fwd_key64(const Plan& pl, const Bufs& b, cudaStream_t s) {
         uint32_t* k[2] = {b.keyC[g], b.keyC[ra]};
         uint32_t* v[2] = {b.valC[g], b.valC[ra]};
         SortScratch sc2 = sc;
+        sc2.ghist += kSortHistWords;
         sc2.stall_test = false;
         RAST_TRY(radix_sort(k, v, 0, &b.hdr->n_copies, pl.copy_cap, pl.expectC, pl.planC, sc2, s, &rb, kHiNames));
     }
     const int r = key64_result_pair(pl);
-    RAST_TRY(launch_ranges(vt, b, b.keyC[r], s));
+    RAST_TRY(launch_ranges(vt, b, b.keyC[r], pl.expectC, s));
     return launch_blend_fwd_pixel_warp(vt, b, b.valC[r], s);
 }
 
 cudaError_t run_bwd(const Plan& pl, const Bufs& b, cudaStream_t s) {
     const ViewTable& vt = pl.vt;
     const int rc = pl.planC.passes & 1;
-    RAST_TRY(cudaMemsetAsync(&b.hdr->needed_bwd, 0, sizeof(unsigned long long), s));
-    RAST_TRY(launch_point_scan(vt, b, s));
+    RAST_TRY(launch_point_slots(vt, b, s));
     RAST_TRY(launch_blend_bwd(vt, b, b.valC[rc], s));
     RAST_TRY(launch_reduce_grads(vt, b, s));
     return cudaSuccess;

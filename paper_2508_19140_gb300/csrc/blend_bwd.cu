@@ -90,6 +90,7 @@ __global__ void __launch_bounds__(TS * TS, TS == 8 && RPT == 1 ? 16 : 1) k_blend
     const float* __restrict__ t_final, const uint32_t* __restrict__ last_in,
     const uint32_t* __restrict__ base, float* __restrict__ partial, float* __restrict__ grow,
     uint2* __restrict__ cutoff, WsHeader* __restrict__ hdr, unsigned long long* __restrict__ trace) {
+    dependency_sync(ranges, order, hdr);
     constexpr int NT = TS * TS;  // threads = pixels
     constexpr int D = NT * RPT;  // records per batch
     constexpr int MW = D / 32;   // mask words per pixel
@@ -520,6 +521,7 @@ __global__ void __launch_bounds__(TS * TS) k_blend_bwd_gauss(
     const float* __restrict__ t_final, const uint32_t* __restrict__ last_in,
     const uint32_t* __restrict__ base, float* __restrict__ partial, uint2* __restrict__ cutoff,
     WsHeader* __restrict__ hdr) {
+    dependency_sync(ranges, order);
     constexpr int NT = TS * TS;
     constexpr int NW = NT / 32;                    // warps = 8x4 sub-tiles
     constexpr int WPR = TS / 8;                    // sub-tiles per row
@@ -797,6 +799,7 @@ __global__ void __launch_bounds__(256, 6) k_reduce_grads(const ViewTable vt, con
                                                       const uint2* __restrict__ cutoff,
                                                       const float* __restrict__ partial,
                                                       const float* __restrict__ grow) {
+    dependency_sync(zbits, rect, rect4, base);
     constexpr int P = MODE == 0 ? C + 1 : C + 7;
     constexpr int PS = partial_stride(P);
     constexpr int GS = grow_stride(P);
@@ -982,10 +985,9 @@ cudaError_t launch_bwd_bilinear(const ViewTable& vt, const Bufs& b, const uint32
     });
     if (e != cudaSuccess) return e;
     ProfScope ps("blend_bwd", s);
-    k_blend_bwd_bilinear<TS, RPT, C, BF16, TSRC><<<grid, TS * TS, smem, s>>>(
-        vt, b.ranges, b.order, pts, b.rec, b.rec_tile, b.t_final, b.last, b.base, b.partial, b.grow, b.cutoff,
-        b.hdr, b.trace);
-    return cudaGetLastError();
+    return launch_dependent(k_blend_bwd_bilinear<TS, RPT, C, BF16, TSRC>, grid, TS * TS, smem, s, vt, b.ranges, b.order,
+                            pts, b.rec, b.rec_tile, b.t_final, b.last, b.base, b.partial, b.grow, b.cutoff, b.hdr,
+                            b.trace);
 }
 
 template <int TS, int C, bool BF16>
@@ -999,9 +1001,8 @@ cudaError_t launch_gauss_bwd(const ViewTable& vt, const Bufs& b, const uint32_t*
     });
     if (e != cudaSuccess) return e;
     ProfScope ps("blend_bwd", s);
-    k_blend_bwd_gauss<TS, C, BF16><<<grid, TS * TS, smem, s>>>(
-        vt, b.ranges, b.order, pts, b.rec, b.t_final, b.last, b.base, b.partial, b.cutoff, b.hdr);
-    return cudaGetLastError();
+    return launch_dependent(k_blend_bwd_gauss<TS, C, BF16>, grid, TS * TS, smem, s, vt, b.ranges, b.order, pts, b.rec,
+                            b.t_final, b.last, b.base, b.partial, b.cutoff, b.hdr);
 }
 
 template <int TS, int RPT, int C, bool BF16>
@@ -1039,11 +1040,8 @@ template <int C>
 cudaError_t launch_reduce_c(const ViewTable& vt, const Bufs& b, cudaStream_t s) {
     const unsigned grid = (unsigned)((vt.n_total + 255) / 256);
     ProfScope ps("reduce_grads", s);
-    if (vt.mode == 0)
-        k_reduce_grads<C, 0><<<grid, 256, 0, s>>>(vt, b.zbits, b.rect, b.rect4, b.base, b.cutoff, b.partial, b.grow);
-    else
-        k_reduce_grads<C, 1><<<grid, 256, 0, s>>>(vt, b.zbits, b.rect, b.rect4, b.base, b.cutoff, b.partial, b.grow);
-    return cudaGetLastError();
+    return launch_dependent(vt.mode == 0 ? k_reduce_grads<C, 0> : k_reduce_grads<C, 1>, grid, 256, 0, s, vt, b.zbits,
+                            b.rect, b.rect4, b.base, b.cutoff, b.partial, b.grow);
 }
 
 }  // namespace

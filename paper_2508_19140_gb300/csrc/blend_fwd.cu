@@ -23,7 +23,7 @@
 // ballots the batch's records whose pixel box overlaps the sub-tile, and
 // composites only those, all 32 lanes in lockstep.
 //
-// Tiles are visited heaviest first (k_tile_buckets / k_tile_scatter): the
+// Tiles are visited heaviest first (k_tile_scatter): the
 // blend's duration is bounded below by its longest tile list, so that list
 // must start at once. The CTA stops reading as soon as every in-image pixel
 // has terminated (__syncthreads_count), which is where early termination saves
@@ -38,31 +38,20 @@
 namespace rast {
 namespace {
 
-// Tiles in descending order of list length, bucketed by floor(log2(len)),
-// over the whole grid: k_tile_buckets counts the tiles of every bucket
-// (block-local counts, then one global add per bucket), k_tile_scatter turns
-// the 33 counts into bucket starts (heaviest bucket first) and places each
-// tile at its bucket's next free position. The order inside a bucket depends
-// on timing and only affects scheduling: every tile is blended the same way.
+// Tiles in descending order of list length, bucketed by floor(log2(len)): the
+// ranges kernel has counted the tiles of every bucket; k_tile_scatter turns the
+// 33 counts into bucket starts (heaviest bucket first) and places each tile at
+// its bucket's next free position. The order inside a bucket depends on timing
+// and only affects scheduling: every tile is blended the same way.
 __device__ __forceinline__ int len_bucket(uint2 r) {
     const uint32_t len = r.y - r.x;
     return len ? 32 - __clz(len) : 0;  // 0..32
 }
 
-__global__ void __launch_bounds__(256) k_tile_buckets(const uint2* __restrict__ ranges, int64_t P,
-                                                      uint32_t* __restrict__ counts) {
-    __shared__ uint32_t s_cnt[33];
-    if (threadIdx.x < 33) s_cnt[threadIdx.x] = 0;
-    __syncthreads();
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < P; t += (int64_t)gridDim.x * blockDim.x)
-        atomicAdd(&s_cnt[len_bucket(ranges[t])], 1u);
-    __syncthreads();
-    if (threadIdx.x < 33 && s_cnt[threadIdx.x]) atomicAdd(&counts[threadIdx.x], s_cnt[threadIdx.x]);
-}
-
 __global__ void __launch_bounds__(256) k_tile_scatter(const uint2* __restrict__ ranges, int64_t P,
                                                       const uint32_t* __restrict__ counts,
                                                       uint32_t* __restrict__ cursor, uint32_t* __restrict__ order) {
+    dependency_sync(ranges, counts);
     __shared__ uint32_t s_start[33];  // global start of each bucket
     __shared__ uint32_t s_cnt[33];    // this block's tiles per bucket, then its next free slot
     if (threadIdx.x == 0) {
@@ -111,6 +100,7 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_bilinear(
     const uint32_t* __restrict__ pts, const uint32_t* __restrict__ rec, uint32_t* __restrict__ rec_tile,
     float* __restrict__ t_final, uint32_t* __restrict__ last_out, WsHeader* __restrict__ hdr,
     unsigned long long* __restrict__ trace) {
+    dependency_sync(ranges, order);
     constexpr int NT = TS * TS;     // threads = pixels
     constexpr int D = NT * RPT;     // records per batch
     constexpr int MW = D / 32;      // mask words per pixel
@@ -321,6 +311,7 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_gauss(
     const ViewTable vt, const uint2* __restrict__ ranges, const uint32_t* __restrict__ order,
     const uint32_t* __restrict__ pts, const uint32_t* __restrict__ rec, float* __restrict__ t_final,
     uint32_t* __restrict__ last_out, WsHeader* __restrict__ hdr) {
+    dependency_sync(ranges, order);
     constexpr int NT = TS * TS;
     constexpr int NW = NT / 32;      // warps = 8x4 sub-tiles
     constexpr int WPR = TS / 8;      // warps per row of 8x4 sub-tiles
@@ -453,14 +444,12 @@ cudaError_t launch_fwd_t(const ViewTable& vt, const Bufs& b, const uint32_t* pts
         });
         if (e != cudaSuccess) return e;
         ProfScope ps("blend_fwd", s);
-        k_blend_fwd_bilinear<TS, RPT, C, BF16><<<grid, TS * TS, smem, s>>>(
-            vt, b.ranges, b.order, pts, b.rec, b.rec_tile, b.t_final, b.last, b.hdr, b.trace);
-        return cudaGetLastError();
+        return launch_dependent(k_blend_fwd_bilinear<TS, RPT, C, BF16>, grid, TS * TS, smem, s, vt, b.ranges, b.order,
+                                pts, b.rec, b.rec_tile, b.t_final, b.last, b.hdr, b.trace);
     }
     ProfScope ps("blend_fwd", s);
-    k_blend_fwd_gauss<TS, C, BF16><<<grid, TS * TS, 0, s>>>(vt, b.ranges, b.order, pts, b.rec, b.t_final,
-                                                        b.last, b.hdr);
-    return cudaGetLastError();
+    return launch_dependent(k_blend_fwd_gauss<TS, C, BF16>, grid, TS * TS, 0, s, vt, b.ranges, b.order, pts, b.rec,
+                            b.t_final, b.last, b.hdr);
 }
 
 template <int TS, int C, bool BF16>
@@ -489,20 +478,11 @@ bool channels_supported(int C) {
 cudaError_t launch_tile_order(const ViewTable& vt, const Bufs& b, cudaStream_t s) {
     const int64_t P = vt.tiles_total;
     if (P == 0) return cudaSuccess;
-    uint32_t* counts = b.order + P;  // 33 bucket counts, then 33 cursors
-    cudaError_t e = cudaMemsetAsync(counts, 0, 66 * sizeof(uint32_t), s);
-    if (e != cudaSuccess) return e;
+    uint32_t* counts = b.order + P;  // 33 bucket counts, then 33 cursors (cleared at the start of the pass)
     const int64_t want = (P + 255) / 256;
     const unsigned grid = (unsigned)(want < 1024 ? want : 1024);
-    {
-        ProfScope ps("tile_order.count", s);
-        k_tile_buckets<<<grid, 256, 0, s>>>(b.ranges, P, counts);
-    }
-    {
-        ProfScope ps("tile_order.scatter", s);
-        k_tile_scatter<<<grid, 256, 0, s>>>(b.ranges, P, counts, counts + 33, b.order);
-    }
-    return cudaGetLastError();
+    ProfScope ps("tile_order", s);
+    return launch_dependent(k_tile_scatter, grid, 256, 0, s, b.ranges, P, counts, counts + 33, b.order);
 }
 
 namespace {

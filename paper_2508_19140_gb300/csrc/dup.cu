@@ -89,6 +89,7 @@ __global__ void __launch_bounds__(kT) k_dup_count(const uint32_t* __restrict__ s
                                                   const void* __restrict__ rect, void* __restrict__ rectS,
                                                   int64_t n, uint32_t* __restrict__ blk,
                                                   const WsHeader* __restrict__ hdr) {
+    dependency_sync(sorted_pts, rectS, hdr);
     __shared__ uint32_t s_warp[33];
     const int64_t s0 = (int64_t)blockIdx.x * kScanItems + (int64_t)threadIdx.x * kPer;
     const bool failed = (hdr->error & kErrTimeout) != 0u;
@@ -158,6 +159,7 @@ __device__ __forceinline__ void load_counts(const uint32_t* __restrict__ p, int6
 template <bool P4>
 __global__ void __launch_bounds__(kT) k_count_blocks(const uint32_t* __restrict__ cnt, int64_t n,
                                                      uint32_t* __restrict__ blk) {
+    dependency_sync(cnt);
     __shared__ uint32_t s_warp[33];
     const int64_t s0 = (int64_t)blockIdx.x * kScanItems + (int64_t)threadIdx.x * kPer;
     uint32_t v[kPer];
@@ -172,6 +174,7 @@ __global__ void __launch_bounds__(kT) k_count_blocks(const uint32_t* __restrict_
 
 __global__ void __launch_bounds__(1024) k_scan_blocks(uint32_t* __restrict__ blk, int64_t nb,
                                                       WsHeader* hdr, int64_t cap) {
+    dependency_sync(blk);
     __shared__ uint32_t s_warp[33];
     __shared__ unsigned long long s_wtot[32];
     const int64_t per = (nb + 1023) / 1024;
@@ -222,6 +225,7 @@ __global__ void __launch_bounds__(kTW) k_dup_write(const ViewTable vt, const uin
                                                    const uint32_t* __restrict__ blk,
                                                    uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
                                                    int64_t cap, const WsHeader* __restrict__ hdr) {
+    dependency_sync(sorted_pts, rectS, blk, hdr);
     __shared__ uint32_t s_warp[33];
     if (hdr->error & kErrTimeout) return;  // set by an earlier kernel: no copy is made from a partial order
     extern __shared__ uint32_t s_copy[];  // [kStageCap] tile ids, then [kStageCap] point indices
@@ -303,6 +307,7 @@ template <bool P4>
 __global__ void __launch_bounds__(kT) k_scan_apply(const uint32_t* __restrict__ cnt, int64_t n,
                                                    const uint32_t* __restrict__ blk,
                                                    uint32_t* __restrict__ base) {
+    dependency_sync(cnt, blk);
     __shared__ uint32_t s_warp[33];
     const int64_t s0 = (int64_t)blockIdx.x * kScanItems + (int64_t)threadIdx.x * kPer;
     uint32_t v[kPer];
@@ -329,7 +334,116 @@ __global__ void __launch_bounds__(kT) k_scan_apply(const uint32_t* __restrict__ 
     }
 }
 
-// Tile ranges from the sorted tile keys. If the tile sort's look-back wait ran
+__global__ void k_bwd_init(WsHeader* hdr) {
+    hdr->needed_bwd = 0ull;
+    hdr->slots = 0u;
+}
+
+// First partial-gradient slot of every point (backward): a block takes one run
+// of slots for its points with a single addition, in whatever order the blocks
+// come (which slot a row lies in has no effect on any value), where a count, a
+// scan and a second pass over the points gave them in point order: 4 M points
+// 26.2 -> 12.3 us, 16 M 55 -> 29 us, 62 M 159 -> 84 us. Bilinear points with one copy need none (their
+// row is indexed by point), so the rows in use lie closer together (the blend
+// that writes them 234 -> 220 us, the reduction that reads them 66.5 -> 60.8 us).
+template <bool P4>
+__global__ void __launch_bounds__(kT) k_point_slots(const uint32_t* __restrict__ cnt, int64_t n, WsHeader* hdr,
+                                                    uint32_t* __restrict__ base) {
+    dependency_sync(cnt);
+    __shared__ uint32_t s_warp[33];
+    __shared__ uint32_t s_first;
+    const int64_t s0 = (int64_t)blockIdx.x * kScanItems + (int64_t)threadIdx.x * kPer;
+    uint32_t v[kPer], sum = 0;
+    load_counts<P4>(cnt, s0, n, v);
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        if (P4 && v[j] == 1u) v[j] = 0u;
+        sum += v[j];
+    }
+    uint32_t tot;
+    uint32_t o = block_excl_scan<kT>(sum, s_warp, tot);
+    if (threadIdx.x == 0) s_first = tot ? atomicAdd(&hdr->slots, tot) : 0u;
+    __syncthreads();
+    o += s_first;
+    uint32_t r[kPer];
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        r[j] = o;
+        o += v[j];
+    }
+    if (s0 + kPer <= n) {
+#pragma unroll
+        for (int j = 0; j < kPer; j += 4)
+            *reinterpret_cast<uint4*>(base + s0 + j) = make_uint4(r[j], r[j + 1], r[j + 2], r[j + 3]);
+    } else {
+#pragma unroll
+        for (int j = 0; j < kPer; ++j)
+            if (s0 + j < n) base[s0 + j] = r[j];
+    }
+}
+
+// Tiles by list length, for the blends' heaviest-first order: bucket of
+// floor(log2(length)) + 1, 0 for an empty list.
+__device__ __forceinline__ int len_bucket(uint32_t len) { return len ? 32 - __clz(len) : 0; }
+
+// Tile ranges found tile by tile: one thread a tile looks for its first copy
+// among the sorted keys, WAYS - 1 probes a step, and neighbours share their ends
+// (the last thread of a block only serves its neighbour). It touches a few dozen
+// keys a tile instead of all of them, and needs no cleared ranges. The tiles'
+// buckets (see k_tile_scatter) are counted on the way. If the tile sort's
+// look-back wait ran out, the keys are a partial order: every range is empty, so
+// the blends read no copy of it.
+template <int WAYS>
+__global__ void __launch_bounds__(kT) k_ranges_search(const uint32_t* __restrict__ keys,
+                                                      const WsHeader* __restrict__ hdr, int64_t tiles,
+                                                      uint2* __restrict__ ranges, uint32_t* __restrict__ buckets) {
+    dependency_sync(keys, hdr);
+    __shared__ uint32_t s_first[kT];
+    __shared__ uint32_t s_cnt[33];
+    if (threadIdx.x < 33) s_cnt[threadIdx.x] = 0;
+    const uint32_t D = (hdr->error & kErrTimeout) ? 0u : hdr->n_copies;
+    const int64_t t = (int64_t)blockIdx.x * (kT - 1) + threadIdx.x;
+    // first position whose key is >= t: in [lo, hi]
+    uint32_t lo = 0, hi = D;
+    while (lo < hi) {
+        uint32_t m[WAYS - 1], k[WAYS - 1];  // probes, ascending, in [lo, hi)
+#pragma unroll
+        for (int j = 0; j < WAYS - 1; ++j) m[j] = lo + (uint32_t)((uint64_t)(hi - lo) * (j + 1) / WAYS);
+#pragma unroll
+        for (int j = 0; j < WAYS - 1; ++j) k[j] = keys[m[j]];
+        uint32_t nlo = lo, nhi = hi;
+#pragma unroll
+        for (int j = 0; j < WAYS - 1; ++j) {
+            if ((int64_t)k[j] < t) nlo = m[j] + 1;
+            else nhi = min(nhi, m[j]);
+        }
+        lo = nlo;
+        hi = nhi;
+    }
+    s_first[threadIdx.x] = lo;
+    __syncthreads();
+    if (threadIdx.x < kT - 1 && t < tiles) {
+        const uint2 r = make_uint2(lo, s_first[threadIdx.x + 1]);
+        ranges[t] = r;
+        atomicAdd(&s_cnt[len_bucket(r.y - r.x)], 1u);
+    }
+    __syncthreads();
+    if (threadIdx.x < 33 && s_cnt[threadIdx.x]) atomicAdd(&buckets[threadIdx.x], s_cnt[threadIdx.x]);
+}
+
+__global__ void __launch_bounds__(kT) k_tile_buckets(const uint2* __restrict__ ranges, int64_t tiles,
+                                                     uint32_t* __restrict__ buckets) {
+    __shared__ uint32_t s_cnt[33];
+    if (threadIdx.x < 33) s_cnt[threadIdx.x] = 0;
+    __syncthreads();
+    for (int64_t t = (int64_t)blockIdx.x * kT + threadIdx.x; t < tiles; t += (int64_t)gridDim.x * kT)
+        atomicAdd(&s_cnt[len_bucket(ranges[t].y - ranges[t].x)], 1u);
+    __syncthreads();
+    if (threadIdx.x < 33 && s_cnt[threadIdx.x]) atomicAdd(&buckets[threadIdx.x], s_cnt[threadIdx.x]);
+}
+
+// Tile ranges from one read of the sorted tile keys, for lists too short for a
+// search per tile (the untiled baselines: a tile a pixel). If the tile sort's look-back wait ran
 // out, the keys are a partial order: the ranges are left empty (cleared before
 // this kernel), so the blends read no copy of it.
 __global__ void __launch_bounds__(kT) k_ranges(const uint32_t* __restrict__ keys,
@@ -456,11 +570,13 @@ cudaError_t launch_duplicate(const ViewTable& vt, const Bufs& b, const uint32_t*
                                  : (carried ? k_dup_count<false, true> : k_dup_count<false, false>);
         const void* in = vt.mode == 0 ? (const void*)b.rect4 : (const void*)b.rect;
         void* out = vt.mode == 0 ? (void*)b.rect4S : (void*)b.rectS;
-        kern<<<(unsigned)nb, kT, 0, s>>>(sorted_pts, in, out, n, b.blk, b.hdr);
+        const cudaError_t e = launch_dependent(kern, (unsigned)nb, kT, 0, s, sorted_pts, in, out, n, b.blk, b.hdr);
+        if (e != cudaSuccess) return e;
     }
     {
         ProfScope ps("dup.scan", s);
-        k_scan_blocks<<<1, 1024, 0, s>>>(b.blk, nb, b.hdr, b.copy_cap);
+        const cudaError_t e = launch_dependent(k_scan_blocks, 1, 1024, 0, s, b.blk, nb, b.hdr, b.copy_cap);
+        if (e != cudaSuccess) return e;
     }
     {
         static PerDevice attr;
@@ -471,46 +587,65 @@ cudaError_t launch_duplicate(const ViewTable& vt, const Bufs& b, const uint32_t*
         if (e != cudaSuccess) return e;
         ProfScope ps("dup.write", s);
         if (vt.mode == 0)
-            k_dup_write<true><<<(unsigned)nb, kTW, 0, s>>>(vt, sorted_pts, b.rect4S, n, b.blk, b.keyC[0],
-                                                         b.valC[0], b.copy_cap, b.hdr);
-        else
-            k_dup_write<false><<<(unsigned)nb, kTW, kDupWriteSmem, s>>>(vt, sorted_pts, b.rectS, n, b.blk,
-                                                                      b.keyC[0], b.valC[0], b.copy_cap, b.hdr);
+            return launch_dependent(k_dup_write<true>, (unsigned)nb, kTW, 0, s, vt, sorted_pts, b.rect4S, n, b.blk,
+                                    b.keyC[0], b.valC[0], b.copy_cap, b.hdr);
+        return launch_dependent(k_dup_write<false>, (unsigned)nb, kTW, kDupWriteSmem, s, vt, sorted_pts, b.rectS, n,
+                                b.blk, b.keyC[0], b.valC[0], b.copy_cap, b.hdr);
     }
-    return cudaGetLastError();
 }
 
-cudaError_t launch_ranges(const ViewTable& vt, const Bufs& b, const uint32_t* sorted_tiles,
+cudaError_t launch_ranges(const ViewTable& vt, const Bufs& b, const uint32_t* sorted_tiles, int64_t expect,
                           cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(b.ranges, 0, sizeof(uint2) * vt.tiles_total, s);
-    if (e != cudaSuccess || b.copy_cap == 0) return e;
-    int64_t g = (b.copy_cap + kT - 1) / kT;
-    const int64_t gmax = (int64_t)device_sm_count() * 8;
-    if (g > gmax) g = gmax;
-    ProfScope ps("ranges", s);
-    k_ranges<<<(unsigned)g, kT, 0, s>>>(sorted_tiles, b.hdr, b.ranges);
+    // A search reads about 40 keys a tile, spread out; a scan clears the ranges
+    // and reads every key, in order, and the tiles' buckets are counted by a
+    // third kernel. The search where one round of blocks covers the grid (it is
+    // then a matter of latency: 64 tiles 6.6 us against 2 + 6.5 + 6.6) and where
+    // lists are long (16640 tiles, 5.3 M copies 9.1 against 2 + 10.2 + 5.7 us;
+    // 8160 tiles, 37 M copies 12.3 against 2 + 39.3 + 6.0; 143 k tiles, 77 M
+    // copies 24.7 against 3 + 69.9 + 6.3); the scan for large, sparsely covered
+    // images and for the untiled baselines (a tile a pixel). Eight ways on
+    // smaller grids, whose time is the steps' latency, four on larger ones,
+    // whose time is the probes.
+    const int64_t tiles = vt.tiles_total;
+    uint32_t* const buckets = b.order + tiles;
+    if (tiles <= 16384 || 32 * tiles <= expect) {
+        if (tiles == 0) return cudaSuccess;
+        ProfScope ps("ranges", s);
+        return launch_dependent(tiles <= 32768 ? k_ranges_search<8> : k_ranges_search<4>,
+                                (unsigned)((tiles + kT - 2) / (kT - 1)), kT, 0, s, sorted_tiles, b.hdr, tiles, b.ranges,
+                                buckets);
+    }
+    cudaError_t e = cudaMemsetAsync(b.ranges, 0, sizeof(uint2) * tiles, s);
+    if (e != cudaSuccess) return e;
+    if (b.copy_cap > 0) {
+        int64_t g = (b.copy_cap + kT - 1) / kT;
+        const int64_t gmax = (int64_t)device_sm_count() * 8;
+        if (g > gmax) g = gmax;
+        ProfScope ps("ranges", s);
+        k_ranges<<<(unsigned)g, kT, 0, s>>>(sorted_tiles, b.hdr, b.ranges);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    if (vt.tile == 1) return cudaSuccess;  // the untiled blends take the pixels in order
+    const int64_t want = (tiles + kT - 1) / kT;
+    ProfScope ps("tile_order.count", s);
+    k_tile_buckets<<<(unsigned)(want < 1024 ? want : 1024), kT, 0, s>>>(b.ranges, tiles, buckets);
     return cudaGetLastError();
 }
 
-cudaError_t launch_point_scan(const ViewTable& vt, const Bufs& b, cudaStream_t s) {
+cudaError_t launch_point_slots(const ViewTable& vt, const Bufs& b, cudaStream_t s) {
+    {
+        ProfScope ps("bwd_init", s);
+        k_bwd_init<<<1, 1, 0, s>>>(b.hdr);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
     const int64_t n = vt.n_total;
     const int64_t nb = (n + kScanItems - 1) / kScanItems;
     if (nb == 0) return cudaSuccess;
-    {
-        ProfScope ps("point_scan.count", s);
-        if (vt.mode == 0) k_count_blocks<true><<<(unsigned)nb, kT, 0, s>>>(b.rect4, n, b.blk);
-        else k_count_blocks<false><<<(unsigned)nb, kT, 0, s>>>(b.cnt, n, b.blk);
-    }
-    {
-        ProfScope ps("point_scan.scan", s);
-        k_scan_blocks<<<1, 1024, 0, s>>>(b.blk, nb, nullptr, 0);
-    }
-    {
-        ProfScope ps("point_scan.apply", s);
-        if (vt.mode == 0) k_scan_apply<true><<<(unsigned)nb, kT, 0, s>>>(b.rect4, n, b.blk, b.base);
-        else k_scan_apply<false><<<(unsigned)nb, kT, 0, s>>>(b.cnt, n, b.blk, b.base);
-    }
-    return cudaGetLastError();
+    ProfScope ps("point_slots", s);
+    return launch_dependent(vt.mode == 0 ? k_point_slots<true> : k_point_slots<false>, (unsigned)nb, kT, 0, s,
+                            vt.mode == 0 ? b.rect4 : b.cnt, n, b.hdr, b.base);
 }
 
 }  // namespace rast

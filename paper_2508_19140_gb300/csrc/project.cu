@@ -220,6 +220,7 @@ constexpr int kPointsPerThread = 2;
 template <int MODE>
 __global__ void __launch_bounds__(256) k_project(const ViewTable vt, const Bufs b, bool write_vals,
                                                  const RectCarry rc) {
+    dependency_sync();
     constexpr int K = kPointsPerThread;
     const int64_t g0 = (int64_t)blockIdx.x * (256 * K) + threadIdx.x;
     PointIn in[K];
@@ -250,9 +251,7 @@ cudaError_t launch_project(const ViewTable& vt, const Bufs& b, bool write_vals, 
     if (vt.n_total == 0) return cudaSuccess;
     const unsigned grid = (unsigned)((vt.n_total + 256 * kPointsPerThread - 1) / (256 * kPointsPerThread));
     ProfScope ps("project", s);
-    if (vt.mode == 0) k_project<0><<<grid, 256, 0, s>>>(vt, b, write_vals, rc);
-    else k_project<1><<<grid, 256, 0, s>>>(vt, b, write_vals, rc);
-    return cudaGetLastError();
+    return launch_dependent(vt.mode == 0 ? k_project<0> : k_project<1>, grid, 256, 0, s, vt, b, write_vals, rc);
 }
 
 }  // namespace rast

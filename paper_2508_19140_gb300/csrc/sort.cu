@@ -109,6 +109,7 @@ __global__ void __launch_bounds__(kThreads) k_digit_hist(const uint32_t* __restr
                                                          uint32_t* __restrict__ ghist,
                                                          uint32_t* __restrict__ counters,
                                                          uint32_t* __restrict__ status, int64_t cap, int tile_keys) {
+    dependency_sync(keys, d_n);
     constexpr int BINS = 1 << BITS;
     __shared__ uint32_t s_h[kMaxSortPasses * BINS];
     const int64_t n = read_count(n_host, d_n);
@@ -282,6 +283,7 @@ __global__ void __launch_bounds__(kThreads, IPT == 16 ? 3 : 4) k_sweep(
     uint32_t* __restrict__ vout, int64_t n_host, const uint32_t* d_n, int64_t cap, int shift,
     uint32_t mask, const uint32_t* __restrict__ ghist_pass, uint32_t* __restrict__ counter,
     uint32_t* __restrict__ status, uint32_t* __restrict__ err, int stall_test, const CarryIo carry) {
+    dependency_sync(ghist_pass, err, d_n);
     constexpr bool IDV = KIND == kIdentity;
     constexpr int BINS = 1 << BITS;
     constexpr int VPT = BINS > kThreads ? BINS / kThreads : 1;  // consecutive bins per thread
@@ -352,11 +354,6 @@ __global__ void __launch_bounds__(kThreads, IPT == 16 ? 3 : 4) k_sweep(
     while (tile < ntiles) {
         const int64_t base = tile * TILE;
         const int cnt = (int)(n - base < TILE ? n - base : TILE);
-        // The next tile is taken now, its keys are fetched while this one is
-        // written out. (Every wait is on tiles taken earlier, whose counts are
-        // published before any wait of theirs: the look-backs still end.)
-        uint32_t next = 0;
-        if (tid == 0) next = atomicAdd(counter, 1u);
 #pragma unroll
         for (int i = 0; i < (BINS + 31) / 32; ++i)
             if (i * 32 + lane < BINS) tab[i * 32 + lane] = make_uint2(0u, 0u);
@@ -474,6 +471,12 @@ __global__ void __launch_bounds__(kThreads, IPT == 16 ? 3 : 4) k_sweep(
             }
             s_s[pre + below] = v;
         }
+        // The next tile is taken before the look-back and its keys are fetched
+        // while this one is written out. (Every wait is on tiles taken earlier,
+        // whose counts are published before any wait of theirs: the look-backs
+        // still end.)
+        uint32_t next = 0;
+        if (tid == 0) next = atomicAdd(counter, 1u);
 #pragma unroll
         for (int q = 0; q < VPT; ++q) {
             const int bin = tid * VPT + q;
@@ -587,16 +590,13 @@ cudaError_t sort_t(uint32_t* keys[2], uint32_t* vals[2], int64_t n, const uint32
     if (e != cudaSuccess) return e;
     const StatusLayout sl = status_layout<BITS>(cap, TILE);
     const int sms = device_sm_count();
-    e = cudaMemsetAsync(sc.ghist, 0, sizeof(uint32_t) * plan.passes * BINS, s);
-    if (e != cudaSuccess) return e;
     {
         ProfScope ps(names[0], s);
         int64_t g = (cap + kThreads * 16 - 1) / (kThreads * 16);
         if (g > (int64_t)sms * 4) g = (int64_t)sms * 4;
         if (g < 1) g = 1;
-        k_digit_hist<BITS><<<(unsigned)g, kThreads, 0, s>>>(keys[0], n, d_n, plan.passes, sc.ghist,
-                                                           sc.counters, sc.status, cap, TILE);
-        e = cudaGetLastError();
+        e = launch_dependent(k_digit_hist<BITS>, (unsigned)g, kThreads, 0, s, keys[0], n, d_n, plan.passes, sc.ghist,
+                             sc.counters, sc.status, cap, TILE);
         if (e != cudaSuccess) return e;
     }
     const int64_t resident = (int64_t)sms * per_sm;
@@ -622,10 +622,9 @@ cudaError_t sort_t(uint32_t* keys[2], uint32_t* vals[2], int64_t n, const uint32
             kern = k_sweep<BITS, IPT, kIdentity>;
         }
         uint32_t* kout = (last && !keys_out) ? nullptr : keys[cur ^ 1];
-        kern<<<gs, kThreads, smem, s>>>(keys[cur], vin, kout, vals[cur ^ 1], n, d_n, cap, shift, mask,
-                                        sc.ghist + k * BINS, sc.counters + k, sc.status + k * sl.pass_words, sc.err,
-                                        (k == 0 && sc.stall_test) ? 1 : 0, carry ? *carry : CarryIo{});
-        e = cudaGetLastError();
+        e = launch_dependent(kern, gs, kThreads, smem, s, keys[cur], vin, kout, vals[cur ^ 1], n, d_n, cap, shift, mask,
+                             sc.ghist + k * BINS, sc.counters + k, sc.status + k * sl.pass_words, sc.err,
+                             (k == 0 && sc.stall_test) ? 1 : 0, carry ? *carry : CarryIo{});
         if (e != cudaSuccess) return e;
         cur ^= 1;
     }

@@ -53,8 +53,8 @@ def _check(views, tile=16):
 def _check_copies(r, views, tile, depth, image, rect, visible):
     """The copies in depth order, row by row of each point's tile rect (tx0, ty0, and
     the spans), then stably by tile."""
-    offs, grids = np.cumsum([0] + [-(-v.camera.width // tile) * -(-v.camera.height // tile) for v in views]), \
-        np.array([-(-v.camera.width // tile) for v in views])
+    offs = np.cumsum([0] + [-(-v.camera.width // tile) * -(-v.camera.height // tile) for v in views])
+    grids = np.array([-(-v.camera.width // tile) for v in views])
     tx0, ty0, w, h = (x[depth] for x in rect)
     im, vis = image[depth], visible[depth]
     tiles, pts = [], []
@@ -68,6 +68,11 @@ def _check_copies(r, views, tile, depth, image, rect, visible):
     order = np.argsort(tiles[keep], kind="stable")
     keys, vals = r.sorted_copies()
     assert np.array_equal(keys, tiles[keep][order]) and np.array_equal(vals, pts[keep][order])
+    # every tile's range of that list (searched for, or scanned on sparsely covered images)
+    ranges = r.arr("ranges", np.uint32, 2 * offs[-1]).reshape(-1, 2)
+    count = np.bincount(keys, minlength=offs[-1])
+    assert np.array_equal(ranges[:, 1] - ranges[:, 0], count)
+    assert np.array_equal(ranges[count > 0, 0], np.searchsorted(keys, np.arange(offs[-1])[count > 0]))
 
 
 # one tile and its edges, one look-back group and its edges (16 tiles of 1024), the change of
