@@ -465,37 +465,10 @@ __device__ __forceinline__ int scatter_index(int lane) {
 constexpr int kGaussBatch = 32;   // records per batch: one ballot per warp and batch
 constexpr int kGaussStages = 4;   // batches staged at once (how far warps may drift apart)
 __host__ __device__ constexpr int gauss_contrib_stride(int P) { return P | 1; }  // odd: conflict-free rows
-// Staged words of a record: the used prefix (u, v, z, o, conic, radius,
-// features) rounded to 16 bytes. A stride of 12 words keeps the lane-parallel
-// reads of the ballot step free of bank conflicts.
-template <int C, bool BF16>
-__host__ __device__ constexpr int gauss_ring_stride() {
-    return (RecLayout<1, C, BF16>::need + 3) & ~3;
-}
 template <int TS, int C, bool BF16>
 constexpr size_t gauss_bwd_smem() {
     return 128 + sizeof(uint32_t) * kGaussStages * kGaussBatch * gauss_ring_stride<C, BF16>() +
            sizeof(float) * kGaussStages * (TS * TS / 32) * kGaussBatch * gauss_contrib_stride(C + 7);
-}
-
-// Polls `bar` for the phase of this parity, giving up after `polls` polls or
-// once another warp of the CTA has given up (abort flag).
-__device__ __forceinline__ bool mbar_wait_or_abort(uint64_t* bar, uint32_t parity, const volatile uint32_t* abort,
-                                                   uint32_t polls) {
-    const uint32_t b = smem_addr(bar);
-    for (uint32_t i = 0; i < polls; ++i) {
-        uint32_t ok;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(ok)
-            : "r"(b), "r"(parity)
-            : "memory");
-        if (ok) return true;
-        if ((i & 63u) == 63u && *abort) return false;
-    }
-    return false;
 }
 
 // The warps of a tile (8x4 sub-tiles) run through the tile's batches without

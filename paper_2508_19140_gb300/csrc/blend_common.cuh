@@ -76,6 +76,10 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
 }
 
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
+}
+
 // Makes the barriers' initialisation visible to the copy engine (follow with
 // a CTA barrier before the first copy).
 __device__ __forceinline__ void mbar_init_fence() {
@@ -133,6 +137,33 @@ struct RecLayout {
 // per-fragment reads of random records conflict less; still a multiple of 16
 // bytes for cp.async.
 __host__ __device__ constexpr int ring_stride(int rw) { return rw + 4; }
+
+// Staged words of a record: the used prefix (u, v, z, o, conic, radius,
+// features) rounded to 16 bytes. A stride of 12 words keeps the lane-parallel
+// reads of the ballot step free of bank conflicts.
+template <int C, bool BF16>
+__host__ __device__ constexpr int gauss_ring_stride() {
+    return (RecLayout<1, C, BF16>::need + 3) & ~3;
+}
+// Polls `bar` for the phase of this parity, giving up after `polls` polls or
+// once another warp of the CTA has given up (abort flag).
+__device__ __forceinline__ bool mbar_wait_or_abort(uint64_t* bar, uint32_t parity, const volatile uint32_t* abort,
+                                                   uint32_t polls) {
+    const uint32_t b = smem_addr(bar);
+    for (uint32_t i = 0; i < polls; ++i) {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(b), "r"(parity)
+            : "memory");
+        if (ok) return true;
+        if ((i & 63u) == 63u && *abort) return false;
+    }
+    return false;
+}
 
 // 128-byte aligned view of a dynamic shared-memory buffer (allocated with
 // 128 spare bytes).
@@ -232,6 +263,23 @@ __device__ __forceinline__ GaussBox gauss_box(float um, float vm, float r) {
     bx.y0 = (int)ceilf(__fsub_rn(vm, r));
     bx.y1 = (int)floorf(__fadd_rn(vm, r));
     return bx;
+}
+
+// The same box as bounds in FP32: an integer p is at least ceil(x) exactly when
+// p >= x, and at most floor(x) when p <= x, so the comparisons decide as with
+// the rounded bounds, without rounding them. (A NaN bound covers no pixel here;
+// its record's distance is NaN as well and excludes every pixel either way.)
+struct GaussBounds {
+    float x0, x1, y0, y1;
+};
+
+__device__ __forceinline__ GaussBounds gauss_bounds(float um, float vm, float r) {
+    return GaussBounds{__fsub_rn(um, r), __fadd_rn(um, r), __fsub_rn(vm, r), __fadd_rn(vm, r)};
+}
+
+// Whether the box meets the pixels [x, x1] x [y, y1].
+__device__ __forceinline__ bool meets(const GaussBounds& b, float x, float x1, float y, float y1) {
+    return b.x0 <= x1 && b.x1 >= x && b.y0 <= y1 && b.y1 >= y;
 }
 
 // Mahalanobis distance squared of pixel (px, py) (FP32, fixed order).

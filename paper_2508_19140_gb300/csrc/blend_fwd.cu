@@ -296,16 +296,33 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_bilinear(
     }
 }
 
-// Gaussian: every warp owns an 8x4 sub-tile and walks the tile's list on its
-// own, 32 records at a time, with no CTA-wide barrier: each lane gathers one
-// record (the CTA's warps read the same records, so all but the first find
-// them in L1), stages it in the warp's own shared-memory rows as three
-// 16-byte words (screen position, opacity and depth; conic; pixel box) plus
-// FP32 features, and the warp ballots the records whose box meets its
-// sub-tile and composites those, all 32 lanes in lockstep. A warp stops as
-// soon as its own 32 pixels have terminated, and never waits for the other
-// sub-tiles of the tile. The next chunk's records are loaded while this one is
-// composited.
+// Gaussian: every warp owns an 8x4 sub-tile and goes through the tile's list
+// with no CTA-wide barrier. The records are staged once for all of the tile's
+// warps, in a ring of kFwdStages batches of kFwdBatch: one warp copies a batch
+// (cp.async) and the batch's mbarrier tells the others when it has landed; the
+// last warp to be done with a batch refills its slot with the batch kFwdStages
+// further on (whose point indices one of the warps has read meanwhile), so warps
+// may drift apart. Of every 32 records a warp ballots those whose box meets the
+// left and the right 4x4 half of its sub-tile, and each half composites its own
+// records, 16 lanes in lockstep, beside the other half's. A warp whose 32 pixels
+// have terminated only keeps count; once all of the tile's warps have, nothing
+// more is staged.
+// Bound by issue slots (86 % busy, about 15 instructions a record and warp).
+// Before, every warp gathered every record itself (three scattered 16-byte loads
+// a record and warp: the L1 pipe 70 % busy) and walked the records that met its
+// whole sub-tile (of 32 records with 3-pixel boxes about 9; a half meets 6): 16 M
+// Gaussians, BF16, 703 -> 566 us; 2 M at 1599x899 397 -> 311 us. Halves alone
+// were 660 and 356 us, the ring with batches of 32 records 611 and 357, of 64
+// 571 and 325 us, of 128 566 and 311 us.
+constexpr int kFwdBatch = 128;
+constexpr int kFwdStages = 3;
+constexpr uint32_t kGaussStop = 2u;  // s_abort: every warp has finished
+
+template <int C, bool BF16>
+constexpr size_t gauss_fwd_smem() {
+    return 128 + sizeof(uint32_t) * kFwdStages * kFwdBatch * gauss_ring_stride<C, BF16>();
+}
+
 template <int TS, int C, bool BF16>
 __global__ void __launch_bounds__(TS * TS) k_blend_fwd_gauss(
     const ViewTable vt, const uint2* __restrict__ ranges, const uint32_t* __restrict__ order,
@@ -315,10 +332,19 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_gauss(
     constexpr int NT = TS * TS;
     constexpr int NW = NT / 32;      // warps = 8x4 sub-tiles
     constexpr int WPR = TS / 8;      // warps per row of 8x4 sub-tiles
-    __shared__ float4 s_a[NW][32];   // (u - 1/2, v - 1/2, opacity, depth)
-    __shared__ float4 s_c[NW][32];   // conic (a, b, c), unused
-    __shared__ int4 s_box[NW][32];   // pixel box (x0, x1, y0, y1)
-    __shared__ __align__(16) float s_f[NW][32 * C];
+    constexpr int GB = kFwdBatch;
+    constexpr int R = kFwdStages;
+    constexpr int NG = GB / 32;      // ballots per batch
+    constexpr int RW = RecLayout<1, C, BF16>::words;
+    constexpr int RS = gauss_ring_stride<C, BF16>();
+    constexpr int FW = RecLayout<1, C, BF16>::feat_word;
+    extern __shared__ __align__(128) uint32_t s_dyn[];
+    uint32_t* const s_ring = align128(s_dyn);      // [R][GB][RS]
+    __shared__ uint32_t s_pnext[R][GB];            // point indices of the batch a slot takes next
+    __shared__ uint32_t s_done[R];                 // warps done with the slot's batch
+    __shared__ __align__(8) uint64_t s_mbar[R];    // slot filled (32 arrivals: the staging lanes)
+    __shared__ uint32_t s_fin;                     // warps whose pixels have all terminated
+    __shared__ uint32_t s_abort;                   // kGaussStop, or 1 after a wait that ran out
     __shared__ uint32_t s_maxstop;
 
     const int64_t tile = order[blockIdx.x];
@@ -327,95 +353,160 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_gauss(
     const int tx = (int)(lt % V.tiles_x), ty = (int)(lt / V.tiles_x);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int sx0 = tx * TS + (warp % WPR) * 8, sy0 = ty * TS + (warp / WPR) * 4;
-    const int px = sx0 + (lane & 7), py = sy0 + (lane >> 3);
+    const int px = sx0 + (lane >> 4) * 4 + (lane & 3), py = sy0 + ((lane >> 2) & 3);
     const bool inside = px < V.W && py < V.H;
     const uint2 rg = ranges[tile];
-    const int RW = vt.rec_words, FW = vt.feat_word;
     const float amax = vt.alpha_max, tmin = vt.t_min;
     const float fpx = (float)px, fpy = (float)py;
-    float4* const wa = s_a[warp];
-    float4* const wc = s_c[warp];
-    int4* const wbox = s_box[warp];
-    float* const wf = s_f[warp];
+    const float fx0 = (float)sx0, fy0 = (float)sy0;
+
+    if (tid < R) {
+        s_done[tid] = 0;
+        mbar_init(&s_mbar[tid], 32);
+    }
+    if (tid == 0) {
+        s_fin = 0;
+        s_abort = 0;
+        s_maxstop = 0;
+    }
+    mbar_init_fence();
+    __syncthreads();
 
     float T = 1.f, A = 0.f, Dp = 0.f;
     float F[C];
 #pragma unroll
     for (int c = 0; c < C; ++c) F[c] = 0.f;
     uint32_t last = 0, stop = 0;
-    bool done = !inside;
-    if (tid == 0) s_maxstop = 0;
+    bool done = !inside, counted = false;
+    const uint32_t nb = (rg.y - rg.x + GB - 1) / GB;
 
-    uint4 g = make_uint4(0u, 0u, 0u, 0u), h = make_uint4(0u, 0u, 0u, 0u);
-    float f[C];
+    // Stages batch j (all 32 lanes of one warp). Batches j >= R take their point
+    // indices from s_pnext.
+    auto stage = [&](uint32_t j) {
+        const int st = (int)(j % R);
 #pragma unroll
-    for (int c = 0; c < C; ++c) f[c] = 0.f;
-    if (rg.x + lane < rg.y) {
-        const uint32_t* rp = rec + (size_t)pts[rg.x + lane] * RW;
-        g = *reinterpret_cast<const uint4*>(rp);
-        h = *reinterpret_cast<const uint4*>(rp + 4);
-        load_features<C, BF16>(rp + FW, f);
+        for (int k = 0; k < NG; ++k) {
+            const uint32_t q = rg.x + j * GB + k * 32 + lane;
+            if (q < rg.y) {
+                const uint32_t gi = j < (uint32_t)R ? pts[q] : s_pnext[st][k * 32 + lane];
+                uint32_t* dst = s_ring + ((size_t)st * GB + k * 32 + lane) * RS;
+                const uint32_t* src = rec + (size_t)gi * RW;
+#pragma unroll
+                for (int w = 0; w < RS; w += 4) cp_async16(dst + w, src + w);
+            }
+        }
+        cp_async_mbar_arrive_noinc(&s_mbar[st]);
+    };
+    if (warp == 0) {
+        for (uint32_t j = 0; j < (uint32_t)R && j < nb; ++j) stage(j);
     }
-    uint32_t gi_next = (rg.x + 32 + lane < rg.y) ? pts[rg.x + 32 + lane] : 0u;
 
+    uint32_t phase = 0;  // parity of the next phase to wait for, per slot
 #pragma unroll 1
-    for (uint32_t q0 = rg.x; q0 < rg.y; q0 += 32) {
-        if (__all_sync(0xffffffffu, done)) break;  // this sub-tile is finished
-        bool hit = false;
-        if (q0 + lane < rg.y) {
-            const float um = __fsub_rn(__uint_as_float(g.x), 0.5f);
-            const float vm = __fsub_rn(__uint_as_float(g.y), 0.5f);
-            const GaussBox bx = gauss_box(um, vm, __uint_as_float(h.w));
-            wa[lane] = make_float4(um, vm, __uint_as_float(g.w), __uint_as_float(g.z));
-            wc[lane] = make_float4(__uint_as_float(h.x), __uint_as_float(h.y), __uint_as_float(h.z), 0.f);
-            wbox[lane] = make_int4(bx.x0, bx.x1, bx.y0, bx.y1);
-            store_row<C>(wf + lane * C, f);
-            hit = bx.x0 <= sx0 + 7 && bx.x1 >= sx0 && bx.y0 <= sy0 + 3 && bx.y1 >= sy0;
+    for (uint32_t j = 0; j < nb; ++j) {
+        const int st = (int)(j % R);
+        const uint32_t fin = __ballot_sync(0xffffffffu, done);
+        if (fin == 0xffffffffu && !counted) {
+            counted = true;
+            if (lane == 0) atomicAdd(&s_fin, 1u);
         }
-        uint32_t m = __ballot_sync(0xffffffffu, hit);
-        __syncwarp();
-        {
-            // the next chunk's record (and the point index of the one after)
-            const uint32_t qn = q0 + 32 + lane;
-            if (qn < rg.y) {
-                const uint32_t* rp = rec + (size_t)gi_next * RW;
-                g = *reinterpret_cast<const uint4*>(rp);
-                h = *reinterpret_cast<const uint4*>(rp + 4);
-                load_features<C, BF16>(rp + FW, f);
+        if (!__all_sync(0xffffffffu, mbar_wait_or_abort(&s_mbar[st], (phase >> st) & 1u, &s_abort, kMbarPolls))) {
+            if (lane == 0 && *(volatile uint32_t*)&s_abort != kGaussStop) {
+                s_abort = 1u;
+                atomicOr(&hdr->error, kErrTimeout);
             }
-            gi_next = (qn + 32 < rg.y) ? pts[qn + 32] : 0u;
+            break;
         }
-        const uint32_t rel0 = q0 - rg.x;
-        while (m) {
-            const int r = __ffs(m) - 1;
-            m &= m - 1;
-            if (done) continue;
-            const int4 bb = wbox[r];
-            if (px < bb.x || px > bb.y || py < bb.z || py > bb.w) continue;
-            const float4 ra = wa[r];
-            const float4 rc = wc[r];
-            const float dx = __fsub_rn(fpx, ra.x), dy = __fsub_rn(fpy, ra.y);
-            const float mm = gauss_m(dx, dy, rc.x, rc.y, rc.z);
-            if (!(mm <= 9.f)) continue;
-            const float alpha = fminf(__fmul_rn(ra.z, gauss_value(mm)), amax);
-            const float nT = __fmul_rn(T, __fsub_rn(1.f, alpha));
-            if (nT < tmin) {
-                done = true;
-                stop = rel0 + r + 1;
-                continue;
-            }
-            float fr[C];
-            load_features<C, false>(reinterpret_cast<const uint32_t*>(wf + r * C), fr);
-            const float ta = T * alpha;
+        if (__any_sync(0xffffffffu, *(volatile uint32_t*)&s_abort == kGaussStop)) break;
+        phase ^= 1u << st;
+        // One warp per batch reads the point indices of batch j + R now and
+        // stores them before it counts itself done.
+        const bool pref = warp == (int)(j % NW) && j + R < nb;
+        uint32_t pnext[NG];
+        if (pref) {
 #pragma unroll
-            for (int c = 0; c < C; ++c) F[c] = fmaf(ta, fr[c], F[c]);
-            Dp = fmaf(ta, ra.w, Dp);
-            A += ta;
-            T = nT;
-            last = rel0 + r + 1;
+            for (int k = 0; k < NG; ++k) {
+                const uint32_t q = rg.x + (j + R) * GB + k * 32 + lane;
+                pnext[k] = q < rg.y ? pts[q] : 0u;
+            }
         }
-        __syncwarp();  // the warp's rows are refilled by the next chunk
+#pragma unroll 1
+        for (int k = 0; k < NG && fin != 0xffffffffu; ++k) {
+            const uint32_t* ring = s_ring + ((size_t)st * GB + k * 32) * RS;
+            const uint32_t rel0 = j * GB + k * 32;
+            bool hit = false, hit2 = false;  // this lane's record meets the left, the right half
+            if (rg.x + rel0 + lane < rg.y) {
+                const uint32_t* rp = ring + lane * RS;
+                const GaussBounds bx = gauss_bounds(__fsub_rn(__uint_as_float(rp[0]), 0.5f),
+                                                    __fsub_rn(__uint_as_float(rp[1]), 0.5f), __uint_as_float(rp[7]));
+                hit = meets(bx, fx0, fx0 + 3.f, fy0, fy0 + 3.f);
+                hit2 = meets(bx, fx0 + 4.f, fx0 + 7.f, fy0, fy0 + 3.f);
+            }
+            const uint32_t left = __ballot_sync(0xffffffffu, hit), right = __ballot_sync(0xffffffffu, hit2);
+            uint32_t m = lane < 16 ? left : right;
+            if (((lane < 16 ? fin : fin >> 16) & 0xffffu) == 0xffffu) m = 0;  // this half has finished
+            __syncwarp();
+            // As many rounds as the longer half has records, all lanes together.
+            const int rounds = max(__popc(__shfl_sync(0xffffffffu, m, 0)), __popc(__shfl_sync(0xffffffffu, m, 16)));
+#pragma unroll 1
+            for (int it = 0; it < rounds; ++it) {
+                const int r = (__ffs(m) - 1) & 31;
+                const bool any = m != 0;
+                m &= m - 1;
+                const uint32_t* rp = ring + r * RS;
+                const uint4 g = *reinterpret_cast<const uint4*>(rp);      // u, v, z, opacity
+                const uint4 h = *reinterpret_cast<const uint4*>(rp + 4);  // conic, radius
+                const float um = __fsub_rn(__uint_as_float(g.x), 0.5f), vm = __fsub_rn(__uint_as_float(g.y), 0.5f);
+                const float dx = __fsub_rn(fpx, um), dy = __fsub_rn(fpy, vm);
+                const float mm = gauss_m(dx, dy, __uint_as_float(h.x), __uint_as_float(h.y), __uint_as_float(h.z));
+                if (any && mm <= 9.f && !done && meets(gauss_bounds(um, vm, __uint_as_float(h.w)), fpx, fpx, fpy, fpy)) {
+                    const float alpha = fminf(__fmul_rn(__uint_as_float(g.w), gauss_value(mm)), amax);
+                    const float nT = __fmul_rn(T, __fsub_rn(1.f, alpha));
+                    if (nT < tmin) {
+                        done = true;
+                        stop = rel0 + r + 1;
+                    } else {
+                        float fr[C];
+                        load_features<C, BF16>(rp + FW, fr);
+                        const float ta = T * alpha;
+#pragma unroll
+                        for (int c = 0; c < C; ++c) F[c] = fmaf(ta, fr[c], F[c]);
+                        Dp = fmaf(ta, __uint_as_float(g.z), Dp);
+                        A += ta;
+                        T = nT;
+                        last = rel0 + r + 1;
+                    }
+                }
+            }
+        }
+        if (pref) {
+#pragma unroll
+            for (int k = 0; k < NG; ++k) s_pnext[st][k * 32 + lane] = pnext[k];
+        }
+        // Done with the batch: the last of the warps refills its slot, unless
+        // every warp has finished.
+        __syncwarp();
+        __threadfence_block();
+        uint32_t prev = 0;
+        if (lane == 0) prev = atomicAdd(&s_done[st], 1u);
+        prev = __shfl_sync(0xffffffffu, prev, 0);
+        if (prev != (uint32_t)(NW - 1)) continue;
+        __threadfence_block();
+        if (__any_sync(0xffffffffu, *(volatile uint32_t*)&s_fin == (uint32_t)NW)) {
+            // Nothing more is blended: warps that wait for the next batch of
+            // this slot (none can wait for a later one) are let through to the flag.
+            if (lane == 0) s_abort = kGaussStop;
+            __syncwarp();
+            __threadfence_block();
+            if (j + R < nb) mbar_arrive(&s_mbar[st]);
+            break;
+        }
+        if (lane == 0) s_done[st] = 0;
+        __syncwarp();
+        __threadfence_block();
+        if (j + R < nb) stage(j + R);
     }
+    cp_async_wait_all();  // no copy may land after the CTA has exited
 
     if (inside) {
         const int64_t pix = (int64_t)py * V.W + px;
@@ -447,8 +538,10 @@ cudaError_t launch_fwd_t(const ViewTable& vt, const Bufs& b, const uint32_t* pts
         return launch_dependent(k_blend_fwd_bilinear<TS, RPT, C, BF16>, grid, TS * TS, smem, s, vt, b.ranges, b.order,
                                 pts, b.rec, b.rec_tile, b.t_final, b.last, b.hdr, b.trace);
     }
+    constexpr size_t smem = gauss_fwd_smem<C, BF16>();
+    static_assert(smem <= 48 * 1024, "within the default dynamic shared memory");
     ProfScope ps("blend_fwd", s);
-    return launch_dependent(k_blend_fwd_gauss<TS, C, BF16>, grid, TS * TS, 0, s, vt, b.ranges, b.order, pts, b.rec,
+    return launch_dependent(k_blend_fwd_gauss<TS, C, BF16>, grid, TS * TS, smem, s, vt, b.ranges, b.order, pts, b.rec,
                             b.t_final, b.last, b.hdr);
 }
 
