@@ -764,20 +764,17 @@ __global__ void __launch_bounds__(TS * TS) k_blend_bwd_gauss(
 
 // ---------------------------------------------------------------- K8 reduce
 
+// The gradients of one point: its copies' rows in rect order, and for Gaussians
+// the chain rule to position and scale.
 template <int C, int MODE>
-__global__ void __launch_bounds__(256, 6) k_reduce_grads(const ViewTable vt, const uint32_t* __restrict__ zbits,
-                                                      const uint2* __restrict__ rect,
-                                                      const uint32_t* __restrict__ rect4,
-                                                      const uint32_t* __restrict__ base,
-                                                      const uint2* __restrict__ cutoff,
-                                                      const float* __restrict__ partial,
-                                                      const float* __restrict__ grow) {
-    dependency_sync(zbits, rect, rect4, base);
+__device__ __forceinline__ void reduce_point(const ViewTable& vt, const uint32_t* __restrict__ zbits,
+                                             const uint2* __restrict__ rect, const uint32_t* __restrict__ rect4,
+                                             const uint32_t* __restrict__ base, const uint2* __restrict__ cutoff,
+                                             const float* __restrict__ partial, const float* __restrict__ grow,
+                                             int64_t gi) {
     constexpr int P = MODE == 0 ? C + 1 : C + 7;
     constexpr int PS = partial_stride(P);
     constexpr int GS = grow_stride(P);
-    const int64_t gi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (gi >= vt.n_total) return;
     const ViewDev& V = vt.v[view_of_point(vt, gi)];
     const int64_t i = gi - V.pt_off;
     float acc[P];
@@ -805,11 +802,11 @@ __global__ void __launch_bounds__(256, 6) k_reduce_grads(const ViewTable vt, con
             return;
         }
     }
-    if (MODE == 0 && cnt) {
-        // Bilinear: one, two or four tiles. The cutoffs of all of them first,
-        // then the rows (two at a time for C <= 11), so a point waits on two
-        // memory round trips rather than two per tile; rows still add up in
-        // rect order.
+    if (cnt && (MODE == 0 || cnt <= 4)) {
+        // At most four tiles (every bilinear point, nearly every small
+        // Gaussian). The cutoffs of all of them first, then the rows (two at a
+        // time for rows of up to 12 floats), so a point waits on two memory
+        // round trips rather than two per tile; rows still add up in rect order.
         const int tx0 = rc.x & 0xffff, ty0 = rc.x >> 16, tx1 = rc.y & 0xffff;
         const int w = tx1 - tx0 + 1;
         bool dn[4];
@@ -821,8 +818,8 @@ __global__ void __launch_bounds__(256, 6) k_reduce_grads(const ViewTable vt, con
                 dn[k] = zb < co.x || (zb == co.x && (uint32_t)gi <= co.y);
             }
         }
-        // A point with one copy has its row indexed by point.
-        const float* pp = cnt == 1 ? grow + (size_t)gi * GS : partial + (size_t)pbase * PS;
+        // A bilinear point with one copy has its row indexed by point.
+        const float* pp = MODE == 0 && cnt == 1 ? grow + (size_t)gi * GS : partial + (size_t)pbase * PS;
         constexpr int KB = PS <= 12 ? 2 : 1;  // rows in flight (wide rows one at a time: no spills)
 #pragma unroll
         for (int k0 = 0; k0 < 4; k0 += KB) {
@@ -855,9 +852,7 @@ __global__ void __launch_bounds__(256, 6) k_reduce_grads(const ViewTable vt, con
                 const uint2 co = cutoff[V.tile_off + (int64_t)ty * V.tiles_x + tx];
                 const bool done = zb < co.x || (zb == co.x && (uint32_t)gi <= co.y);
                 if (!done) continue;
-                // Bilinear points with one copy have their row indexed by point.
-                const bool own = MODE == 0 && cnt == 1;
-                const float4* row = reinterpret_cast<const float4*>(own ? grow + (size_t)gi * GS : pp + (size_t)k * PS);
+                const float4* row = reinterpret_cast<const float4*>(pp + (size_t)k * PS);
 #pragma unroll
                 for (int j = 0; j < PS / 4; ++j) {
                     const float4 x = row[j];
@@ -947,6 +942,93 @@ __global__ void __launch_bounds__(256, 6) k_reduce_grads(const ViewTable vt, con
     if (V.d_scale) V.d_scale[i] = V.scale ? gs : 0.f;
 }
 
+template <int C>
+__global__ void __launch_bounds__(256, 6) k_reduce_grads(const ViewTable vt, const uint32_t* __restrict__ zbits,
+                                                      const uint2* __restrict__ rect,
+                                                      const uint32_t* __restrict__ rect4,
+                                                      const uint32_t* __restrict__ base,
+                                                      const uint2* __restrict__ cutoff,
+                                                      const float* __restrict__ partial,
+                                                      const float* __restrict__ grow) {
+    dependency_sync(zbits, rect, rect4, base);
+    const int64_t gi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (gi >= vt.n_total) return;
+    reduce_point<C, 0>(vt, zbits, rect, rect4, base, cutoff, partial, grow, gi);
+}
+
+// Gaussian points. Behind the early termination of a dense frame most points
+// have no replayed copy (7 of 8 on the 16 M-point frame) and zero gradients:
+// those are written at once, without reading position, scale or rows. The
+// others, scattered over all warps, are collected in shared memory and worked
+// on by full warps: every warp running the chain rule for a few of its lanes
+// took 546 us on that frame (46 % issue-active, 589 instructions a warp), this
+// 349 us. A point also counts as replayed where a factor of the chain may not
+// be finite, so that its product with zero sums is not zero: a scale that is
+// not finite makes the rect cover the whole image, and a covariance may be
+// singular without dilation, or overflow next to the camera.
+template <int C>
+__global__ void __launch_bounds__(256, 4) k_reduce_gauss(const ViewTable vt, const uint32_t* __restrict__ zbits,
+                                                      const uint2* __restrict__ rect,
+                                                      const uint32_t* __restrict__ rect4,
+                                                      const uint32_t* __restrict__ base,
+                                                      const uint2* __restrict__ cutoff,
+                                                      const float* __restrict__ partial,
+                                                      const float* __restrict__ grow) {
+    dependency_sync(zbits, rect, rect4, base);
+    constexpr int K = 4;  // points per thread
+    __shared__ uint16_t s_queue[256 * K];
+    __shared__ uint32_t s_count;
+    if (threadIdx.x == 0) s_count = 0;
+    __syncthreads();
+    const int64_t g0 = (int64_t)blockIdx.x * (256 * K);
+    uint2 rc[K];
+    uint32_t zb[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int64_t gi = g0 + k * 256 + threadIdx.x;
+        rc[k] = gi < vt.n_total ? rect[gi] : make_uint2(1u, 0u);
+        zb[k] = gi < vt.n_total ? zbits[gi] : 0u;
+    }
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int64_t gi = g0 + k * 256 + threadIdx.x;
+        if (gi >= vt.n_total) continue;
+        const ViewDev& V = vt.v[view_of_point(vt, gi)];
+        const int tx0 = rc[k].x & 0xffff, ty0 = rc[k].x >> 16, tx1 = rc[k].y & 0xffff, ty1 = rc[k].y >> 16;
+        const uint32_t cnt = rect_count(rc[k]);
+        bool hit = false;
+        if (cnt) {
+            hit = vt.dilation < 1e-6f || !(__uint_as_float(zb[k]) > 1e-5f) ||
+                  (rc[k].x == 0u && tx1 == V.tiles_x - 1 && ty1 == V.tiles_y - 1);
+            for (int ty = ty0; ty <= ty1 && !hit; ++ty)
+                for (int tx = tx0; tx <= tx1; ++tx) {
+                    const uint2 co = cutoff[V.tile_off + (int64_t)ty * V.tiles_x + tx];
+                    hit = hit || zb[k] < co.x || (zb[k] == co.x && (uint32_t)gi <= co.y);
+                }
+        }
+        if (hit) {
+            s_queue[atomicAdd(&s_count, 1u)] = (uint16_t)(k * 256 + threadIdx.x);
+            continue;
+        }
+        const int64_t i = gi - V.pt_off;
+        float zero[C];
+#pragma unroll
+        for (int c = 0; c < C; ++c) zero[c] = 0.f;
+        if (V.d_feat) store_row<C>(V.d_feat + i * C, zero);
+        if (V.d_opacity) V.d_opacity[i] = 0.f;
+        if (V.d_xyz) {
+            V.d_xyz[3 * i] = 0.f;
+            V.d_xyz[3 * i + 1] = 0.f;
+            V.d_xyz[3 * i + 2] = 0.f;
+        }
+        if (V.d_scale) V.d_scale[i] = 0.f;
+    }
+    __syncthreads();
+    const uint32_t n = s_count;
+    for (uint32_t q = threadIdx.x; q < n; q += 256)
+        reduce_point<C, 1>(vt, zbits, rect, rect4, base, cutoff, partial, grow, g0 + s_queue[q]);
+}
+
 template <int TS, int RPT, int C, bool BF16, bool TSRC>
 cudaError_t launch_bwd_bilinear(const ViewTable& vt, const Bufs& b, const uint32_t* pts, cudaStream_t s) {
     const unsigned grid = (unsigned)vt.tiles_total;
@@ -1011,10 +1093,11 @@ cudaError_t launch_bwd_c(const ViewTable& vt, const Bufs& b, const uint32_t* pts
 
 template <int C>
 cudaError_t launch_reduce_c(const ViewTable& vt, const Bufs& b, cudaStream_t s) {
-    const unsigned grid = (unsigned)((vt.n_total + 255) / 256);
+    const int per = vt.mode == 0 ? 256 : 1024;  // points per block
+    const unsigned grid = (unsigned)((vt.n_total + per - 1) / per);
     ProfScope ps("reduce_grads", s);
-    return launch_dependent(vt.mode == 0 ? k_reduce_grads<C, 0> : k_reduce_grads<C, 1>, grid, 256, 0, s, vt, b.zbits,
-                            b.rect, b.rect4, b.base, b.cutoff, b.partial, b.grow);
+    return launch_dependent(vt.mode == 0 ? k_reduce_grads<C> : k_reduce_gauss<C>, grid, 256, 0, s, vt, b.zbits, b.rect,
+                            b.rect4, b.base, b.cutoff, b.partial, b.grow);
 }
 
 }  // namespace
