@@ -304,15 +304,10 @@ __global__ void __launch_bounds__(TS * TS, TS == 8 && RPT == 1 ? 16 : 1) k_blend
         __syncthreads();
         if (inside && last > rel0) {
             // One loop over the set bits of the pixel's mask, last to first.
-            int w = MW - 1;
-            uint32_t m = s_mask[tid][MW - 1];
+            MaskWalk<MW, false> walk(s_mask[tid]);
 #pragma unroll 1
-            while (true) {
-                while (m == 0 && w > 0) m = s_mask[tid][--w];
-                if (m == 0) break;
-                const int bit = 31 - __clz(m);
-                m &= ~(1u << bit);
-                const int r = w * 32 + bit;
+            while (walk.more()) {
+                const int r = walk.next();
                 if (rel0 + r >= last) continue;
                 const float2 wi = my_wi[4 * r];
                 const float2 oz = s_oz[r];

@@ -227,6 +227,65 @@ __device__ __forceinline__ void load_features(const uint32_t* __restrict__ rp, f
     }
 }
 
+// Walk over the set bits of a pixel's batch mask (MW words, in shared memory),
+// ascending or descending. Two words stay in registers as one; of more, only
+// those that are not empty are taken, the next one already loaded (a loop over
+// empty words costs every lane of the warp the longest lane's steps, a load at
+// the change of words its latency). Against a scanning loop, forward / backward:
+// 16x16 tiles, 20 k points 57 -> 54 us, 60 k 41 -> 37 / 44 -> 42, 500 k 94 -> 83,
+// 8 M 258 -> 222; 8x8 tiles, 4 M 128 -> 121 / 220 -> 211.
+template <int MW, bool UP>
+struct MaskWalk {
+    const uint32_t* row;
+    uint32_t m, next_m, rest;  // bits left in the current word; the next word; words after it
+    int w, next_w;
+
+    __device__ __forceinline__ void prefetch() {
+        next_m = 0;
+        if (rest) {
+            next_w = UP ? __ffs(rest) - 1 : 31 - __clz(rest);
+            rest &= ~(1u << next_w);
+            next_m = row[next_w];
+        }
+    }
+
+    __device__ __forceinline__ explicit MaskWalk(const uint32_t* row_) : row(row_) {
+        rest = 0;
+#pragma unroll
+        for (int k = 0; k < MW; ++k) rest |= row[k] ? 1u << k : 0u;
+        next_w = 0;
+        prefetch();
+        m = next_m;
+        w = next_w;
+        prefetch();
+    }
+
+    // Whether bits are left; next() takes one.
+    __device__ __forceinline__ bool more() const { return (m | next_m) != 0u; }
+    __device__ __forceinline__ int next() {
+        if (m == 0) {
+            m = next_m;
+            w = next_w;
+            prefetch();
+        }
+        const int b = UP ? __ffs(m) - 1 : 31 - __clz(m);
+        m &= ~(1u << b);
+        return w * 32 + b;
+    }
+};
+
+template <bool UP>
+struct MaskWalk<2, UP> {
+    unsigned long long m;
+    __device__ __forceinline__ explicit MaskWalk(const uint32_t* row) : m(row[0] | (unsigned long long)row[1] << 32) {}
+    __device__ __forceinline__ bool more() const { return m != 0ull; }
+    __device__ __forceinline__ int next() {
+        const int b = UP ? __ffsll(m) - 1 : 63 - __clzll(m);
+        m &= ~(1ull << b);
+        return b;
+    }
+};
+
 // Bilinear anchor and fractions from the screen position (exact in FP32).
 struct BilinGeom {
     int i0, j0;

@@ -229,14 +229,10 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_bilinear(
         if (__syncthreads_count(!done) == 0) break;
         if (!done) {
             // One loop over every set bit of the pixel's D-bit mask, in order.
-            int w = 0;
-            uint32_t m = s_mask[tid][0];
+            MaskWalk<MW, true> walk(s_mask[tid]);
 #pragma unroll 1
-            while (true) {
-                while (m == 0 && w < MW - 1) m = s_mask[tid][++w];
-                if (m == 0) break;
-                const int r = w * 32 + __ffs(m) - 1;
-                m &= m - 1;
+            while (walk.more()) {
+                const int r = walk.next();
                 const float alpha = my_alpha[4 * r];
                 const float z = s_z[r];
                 const float nT = __fmul_rn(T, __fsub_rn(1.f, alpha));
