@@ -211,13 +211,16 @@ __global__ void __launch_bounds__(1024) k_scan_blocks(uint32_t* __restrict__ blk
 constexpr int kTW = 2 * kT;
 constexpr int kPerW = kScanItems / kTW;
 static_assert(kPerW == 4, "the packed-rect path loads four rects as one 16-byte vector");
-// Gaussian copies a block stages in shared memory before writing them out
-// (four a point on average fit; a block with more writes its copies
-// directly). Bilinear points make at most four copies each, in runs of one
-// to four per thread, and write them directly: measured, staging them costs
-// more occupancy than the scattered stores do.
-constexpr int kStageCap = 4 * kScanItems;
-constexpr size_t kDupWriteSmem = sizeof(uint32_t) * 2 * kStageCap;
+// Copies a block stages in shared memory before writing them out in coalesced
+// runs (a block with more writes them directly): four a point for Gaussians
+// (about two on average), one and a half for bilinear points (1.1 to 1.3), whose
+// one, two or four copies are written without loops: 4 M points 38 -> 25 us, 32 M
+// 203 -> 145 us, 62 M in 8 images 483 -> 381 us (staging alone, behind the loops,
+// was 34, 219 and 512 us, direct stores without loops 39, 209 and 439 us).
+template <bool P4>
+constexpr int stage_cap() { return P4 ? 3 * kScanItems / 2 : 4 * kScanItems; }
+template <bool P4>
+constexpr size_t dup_write_smem() { return sizeof(uint32_t) * 2 * stage_cap<P4>(); }
 
 template <bool P4>
 __global__ void __launch_bounds__(kTW) k_dup_write(const ViewTable vt, const uint32_t* __restrict__ sorted_pts,
@@ -271,24 +274,47 @@ __global__ void __launch_bounds__(kTW) k_dup_write(const ViewTable vt, const uin
     // The block's copies fill one contiguous range of the output: staged in
     // shared memory, they leave in coalesced runs instead of one scattered
     // 4-byte store per copy and array.
-    const bool staged = !P4 && tot <= (uint32_t)kStageCap;
+    constexpr int kStageCap = stage_cap<P4>();
+    const bool staged = tot <= (uint32_t)kStageCap;
     uint32_t o = staged ? ex : blk0 + ex;
 #pragma unroll
     for (int j = 0; j < kPerW; ++j) {
         if (c[j] == 0) continue;
         const ViewDev& V = vt.v[view_of_point(vt, gi[j])];
         const int tx0 = r[j].x & 0xffff, ty0 = r[j].x >> 16, tx1 = r[j].y & 0xffff, ty1 = r[j].y >> 16;
-        for (int ty = ty0; ty <= ty1; ++ty) {
-            const uint32_t row = (uint32_t)(V.tile_off + (int64_t)ty * V.tiles_x);
-            for (int tx = tx0; tx <= tx1; ++tx) {
+        if constexpr (P4) {
+            // at most two by two tiles: no loops
+            auto put = [&](uint32_t at, uint32_t tile, uint32_t g) {
                 if (staged) {
-                    s_copy[o] = row + (uint32_t)tx;
-                    s_copy[kStageCap + o] = gi[j];
-                } else if ((int64_t)o < cap) {
-                    keys[o] = row + (uint32_t)tx;
-                    vals[o] = gi[j];
+                    s_copy[at] = tile;
+                    s_copy[kStageCap + at] = g;
+                } else if ((int64_t)at < cap) {
+                    keys[at] = tile;
+                    vals[at] = g;
                 }
-                ++o;
+            };
+            const uint32_t tiles_x = (uint32_t)V.tiles_x, w = (uint32_t)(tx1 - tx0);
+            const uint32_t first = (uint32_t)V.tile_off + (uint32_t)ty0 * tiles_x + (uint32_t)tx0;
+            put(o, first, gi[j]);
+            if (w) put(o + 1, first + 1, gi[j]);
+            if (ty1 != ty0) {
+                put(o + 1 + w, first + tiles_x, gi[j]);
+                if (w) put(o + 3, first + tiles_x + 1, gi[j]);
+            }
+            o += c[j];
+        } else {
+            for (int ty = ty0; ty <= ty1; ++ty) {
+                const uint32_t row = (uint32_t)(V.tile_off + (int64_t)ty * V.tiles_x);
+                for (int tx = tx0; tx <= tx1; ++tx) {
+                    if (staged) {
+                        s_copy[o] = row + (uint32_t)tx;
+                        s_copy[kStageCap + o] = gi[j];
+                    } else if ((int64_t)o < cap) {
+                        keys[o] = row + (uint32_t)tx;
+                        vals[o] = gi[j];
+                    }
+                    ++o;
+                }
             }
         }
     }
@@ -582,14 +608,16 @@ cudaError_t launch_duplicate(const ViewTable& vt, const Bufs& b, const uint32_t*
         static PerDevice attr;
         const cudaError_t e = per_device(attr, nullptr, [](int, int*) {
             return cudaFuncSetAttribute(k_dup_write<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)kDupWriteSmem);
+                                        (int)dup_write_smem<false>());
         });
         if (e != cudaSuccess) return e;
         ProfScope ps("dup.write", s);
         if (vt.mode == 0)
-            return launch_dependent(k_dup_write<true>, (unsigned)nb, kTW, 0, s, vt, sorted_pts, b.rect4S, n, b.blk,
+            return launch_dependent(k_dup_write<true>, (unsigned)nb, kTW, dup_write_smem<true>(), s, vt, sorted_pts,
+                                    b.rect4S, n, b.blk,
                                     b.keyC[0], b.valC[0], b.copy_cap, b.hdr);
-        return launch_dependent(k_dup_write<false>, (unsigned)nb, kTW, kDupWriteSmem, s, vt, sorted_pts, b.rectS, n,
+        return launch_dependent(k_dup_write<false>, (unsigned)nb, kTW, dup_write_smem<false>(), s, vt, sorted_pts,
+                                b.rectS, n,
                                 b.blk, b.keyC[0], b.valC[0], b.copy_cap, b.hdr);
     }
 }
