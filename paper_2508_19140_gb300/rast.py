@@ -194,12 +194,8 @@ def make_camera(cam) -> Camera:
     """From any object with fx, fy, cx, cy, R (3x3), t (3), width, height, near, far."""
     c = Camera()
     c.fx, c.fy, c.cx, c.cy = float(cam.fx), float(cam.fy), float(cam.cx), float(cam.cy)
-    R = np.asarray(cam.R, np.float32).reshape(9)
-    t = np.asarray(cam.t, np.float32).reshape(3)
-    for k in range(9):
-        c.R[k] = float(R[k])
-    for k in range(3):
-        c.t[k] = float(t[k])
+    c.R[:] = np.asarray(cam.R, np.float32).reshape(9).tolist()
+    c.t[:] = np.asarray(cam.t, np.float32).reshape(3).tolist()
     c.near_z = float(getattr(cam, "near", 0.2))
     c.far_z = float(getattr(cam, "far", 1e4))
     c.width, c.height = int(cam.width), int(cam.height)
@@ -252,7 +248,9 @@ def make_grads(g_feat, g_alpha=None, g_depth=None, d_feat=None, d_opacity=None, 
 
 def _stream(stream):
     if stream is None:
-        stream = torch.cuda.current_stream()
+        # the current stream's handle, without building a Stream object (three
+        # calls a training step: about 8 us each)
+        return ct.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
     return ct.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
 
 
@@ -490,7 +488,9 @@ class _Batch(torch.autograd.Function):
             st, stats = rasterize_get_status(ws)
             if st != RAST_OK:
                 raise RastError(st, f"rasterize forward ({stats})")
-        ctx.cams, ctx.opts_kw, ctx.n_views = cams, opts_kw, n_views
+        # The marshalled options and cameras serve the backward as well: the
+        # pair of passes sees one camera each.
+        ctx.opts, ctx.c_cams, ctx.n_views = opts, [v.cam for v in views], n_views
         ctx.save_for_backward(ws, *[t for p in pts for t in p if t is not None])
         ctx.has_scale = [p[3] is not None for p in pts]
         ctx.feat_dtypes = [p[2].dtype for p in pts]
@@ -501,7 +501,7 @@ class _Batch(torch.autograd.Function):
         saved = ctx.saved_tensors
         ws = saved[0]
         it = iter(saved[1:])
-        opts = make_opts(**ctx.opts_kw)
+        opts = ctx.opts
         gauss = opts.mode == GAUSSIAN
         dev = ws.device
         views, grads_out = [], []
@@ -510,7 +510,7 @@ class _Batch(torch.autograd.Function):
             scale = next(it) if ctx.has_scale[k] else None
             gF, gA, gD = gouts[3 * k: 3 * k + 3]
             if gF is None:
-                gF = torch.zeros((ctx.cams[k].height, ctx.cams[k].width, feat.shape[1]),
+                gF = torch.zeros((ctx.c_cams[k].height, ctx.c_cams[k].width, feat.shape[1]),
                                  dtype=torch.float32, device=dev)
             else:
                 gF = gF.contiguous().float()
@@ -523,7 +523,7 @@ class _Batch(torch.autograd.Function):
             d_scale = torch.empty((n,), dtype=torch.float32, device=dev) if (gauss and scale is not None) else None
             v = View()
             v.pts = make_points(xyz, op, feat, scale)
-            v.cam = make_camera(ctx.cams[k])
+            v.cam = ctx.c_cams[k]
             v.grad = make_grads(gF, gA, gD, d_feat, d_op, d_xyz, d_scale)
             views.append(v)
             grads_out.append([d_xyz, d_op, d_feat, d_scale])
