@@ -182,21 +182,23 @@ def kernel_bytes(name, w):
     if name.endswith(".hist"):      # one read of the keys counts every pass's digits
         return 4 * (N if name.startswith("depth") else D)
     if name.endswith(".sweep"):     # per pass: read key+value, write key+value
-        if name.startswith("depth"):  # the first pass makes the point indices itself
+        if name.startswith("depth"):
+            # the first pass reads the points' rects for the values it makes, the
+            # last writes them in place of the keys
             passes = max(w.get("depth_passes", 1), 1)
-            return (16 * passes - 4) * N / passes
+            return (16 * passes + rb - 4) * N / passes
         return 16 * D
-    if name == "dup.count":   # sorted point indices, gathered rects, rects in depth order
+    if name == "dup.count":   # rects in depth order (carried by the depth sort)
+        return N * rb
+    if name == "dup.gather":  # frames whose rects are not carried: indices, rects, rects in depth order
         return N * (4 + rb + rb)
     if name == "dup.write":
         return N * (rb + 4) + D * 8
-    if name == "ranges":
-        return D * 4 + P * 8
+    if name == "ranges":      # a search of about 40 keys a tile
+        return P * (8 + 4 * 40)
     if name == "blend_fwd":
         return Dn * (rec + 4) + P * 8 + HW * (4 * C + 16)
-    if name == "point_scan.count":
-        return N * 4
-    if name == "point_scan.apply":
+    if name == "point_slots":
         return N * 8
     if name == "blend_bwd":   # replayed records + indices, one gradient row per copy, pixel state
         return Db * (rec + 4 + 4 * npart) + P * 16 + HW * (4 * C + 16)

@@ -108,7 +108,7 @@ typedef struct {
 
 /* Test hook for the bounded device-side waits (failure detection). With this
  * flag the first digit pass of the depth sort withholds the look-back word of
- * its first 4096-key tile, so the tile after it waits on a word nothing will
+ * its first tile of keys, so the tile after it waits on a word nothing will
  * ever set, and that wait is limited to 64 polls instead of 2^22. The wait
  * runs out, the kernel sets the timeout bit of the workspace error word and
  * returns normally; every later stage sees the bit and produces an empty copy

@@ -463,7 +463,7 @@ const char* const kTileSortNames[2] = {"tile_sort.hist", "tile_sort.sweep"};
 
 cudaError_t launch_init(const Plan& pl, const Bufs& b, cudaStream_t s) {
     const ViewTable& vt = pl.vt;
-    ProfScope ps("init", s);
+    ProfScope ps("init_header", s);
     k_init<<<1, 1024, 0, s>>>(b.hdr, vt.n_views, vt.n_total, pl.copy_cap, vt.tiles_total, vt.pix_total,
                               pl.save_tiled ? 1u : 0u, b.sort_ghist, b.order + vt.tiles_total);
     return cudaGetLastError();

@@ -20,8 +20,9 @@
 // in ascending order = list order.
 //
 // Gaussian splats cover many pixels; there each warp owns an 8x4 sub-tile,
-// ballots the batch's records whose pixel box overlaps the sub-tile, and
-// composites only those, all 32 lanes in lockstep.
+// ballots the records whose pixel box meets its two 4x4 halves, and each half
+// composites its own, 16 lanes in lockstep; the records are staged once for the
+// tile's warps, which run through them without CTA barriers.
 //
 // Tiles are visited heaviest first (k_tile_scatter): the
 // blend's duration is bounded below by its longest tile list, so that list
@@ -570,7 +571,7 @@ cudaError_t launch_tile_order(const ViewTable& vt, const Bufs& b, cudaStream_t s
     uint32_t* counts = b.order + P;  // 33 bucket counts, then 33 cursors (cleared at the start of the pass)
     const int64_t want = (P + 255) / 256;
     const unsigned grid = (unsigned)(want < 1024 ? want : 1024);
-    ProfScope ps("tile_order", s);
+    ProfScope ps("tile_order.scatter", s);
     return launch_dependent(k_tile_scatter, grid, 256, 0, s, b.ranges, P, counts, counts + 33, b.order);
 }
 
