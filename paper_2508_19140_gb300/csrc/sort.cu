@@ -336,7 +336,8 @@ __device__ __forceinline__ void carry_unpack(const RectCarry& rc, uint32_t k, ui
 // turn 151 us a pass over 32 M keys. Three CTAs on an SM (80 registers, 57 KB)
 // with the next tile on its way beat four without: 147 us. The whole pass went
 // 217 -> 147 us (32 M keys, 7-bit digits; 3.6 TB/s moved), 36.6 -> 27 us (4 M
-// keys), 433 -> 308 us (62 M keys, 8-bit), 630 -> 535 us (77 M keys, 9-bit).
+// keys), 433 -> 322 us (62 M keys, 8-bit), 630 -> 493 us (77 M keys, 9-bit; a thread's
+// two bins 256 apart: 553 us with neighbouring ones, whose counters share banks).
 template <int BITS, int IPT, int KIND>
 __global__ void __launch_bounds__(kThreads, IPT == 16 ? 3 : 4) k_sweep(
     const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint32_t* __restrict__ kout,
@@ -346,7 +347,7 @@ __global__ void __launch_bounds__(kThreads, IPT == 16 ? 3 : 4) k_sweep(
     dependency_sync(ghist_pass, err, d_n);
     constexpr bool IDV = KIND == kIdentity;
     constexpr int BINS = 1 << BITS;
-    constexpr int VPT = BINS > kThreads ? BINS / kThreads : 1;  // consecutive bins per thread
+    constexpr int VPT = BINS > kThreads ? BINS / kThreads : 1;  // bins per thread: tid, tid + kThreads
     constexpr int TILE = kThreads * IPT;
     extern __shared__ __align__(128) uint32_t s_dyn[];
     uint32_t* s_k = align128(s_dyn);  // TILE: the tile's keys, then its keys in digit order
@@ -390,21 +391,14 @@ __global__ void __launch_bounds__(kThreads, IPT == 16 ? 3 : 4) k_sweep(
     }
     // Global start of every digit in this pass.
     {
-        uint32_t tot[VPT];
-        uint32_t local = 0;
+        uint32_t before = 0;
 #pragma unroll
         for (int q = 0; q < VPT; ++q) {
-            const int bin = tid * VPT + q;
-            tot[q] = bin < BINS ? ghist_pass[bin] : 0u;
-            local += tot[q];
-        }
-        uint32_t all;
-        uint32_t ex = block_excl_scan<kThreads>(local, s_warp, all);
-#pragma unroll
-        for (int q = 0; q < VPT; ++q) {
-            const int bin = tid * VPT + q;
-            if (bin < BINS) s_goff[bin] = ex;
-            ex += tot[q];
+            const int bin = tid + q * kThreads;
+            uint32_t all;
+            const uint32_t ex = block_excl_scan<kThreads>(bin < BINS ? ghist_pass[bin] : 0u, s_warp, all);
+            if (bin < BINS) s_goff[bin] = before + ex;
+            before += all;
         }
     }
     __syncthreads();
@@ -444,10 +438,10 @@ __global__ void __launch_bounds__(kThreads, IPT == 16 ? 3 : 4) k_sweep(
         const bool publish = ntiles > 1 && !(stall_test && tile == 0);
         uint32_t tot[VPT];           // the tile's count of this thread's bins, keys past the end left out
         uint32_t c[VPT][kWarps];     // each warp's count
-        uint32_t local = 0;          // all of them
+        uint32_t local[VPT], inc[VPT];  // all of them, and their sums over the warp's lanes
 #pragma unroll
         for (int q = 0; q < VPT; ++q) {
-            const int bin = tid * VPT + q;
+            const int bin = tid + q * kThreads;
             uint32_t sum = 0;
             if (bin < BINS) {
 #pragma unroll
@@ -461,18 +455,22 @@ __global__ void __launch_bounds__(kThreads, IPT == 16 ? 3 : 4) k_sweep(
                     atomicAdd(&groups[(tile / kGroup) * BINS + bin].y, kArrival | tot[q]);
                 }
             }
-            local += sum;
+            local[q] = sum;
+            inc[q] = warp_incl_scan(sum);
+            if (lane == 31) s_warp[q * kWarps + warp] = inc[q];
         }
-        const uint32_t inc = warp_incl_scan(local);
-        if (lane == 31) s_warp[warp] = inc;
         __syncthreads();
-        uint32_t run = inc - local;
-#pragma unroll
-        for (int w = 0; w < kWarps - 1; ++w) run += w < warp ? s_warp[w] : 0u;
-        uint32_t start[VPT];
+        uint32_t start[VPT], before = 0;
 #pragma unroll
         for (int q = 0; q < VPT; ++q) {
-            const int bin = tid * VPT + q;
+            const int bin = tid + q * kThreads;
+            uint32_t run = before + inc[q] - local[q];
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) {
+                const uint32_t x = s_warp[q * kWarps + w];
+                run += w < warp ? x : 0u;
+                before += x;
+            }
             start[q] = run;
             if (bin < BINS) {
 #pragma unroll
@@ -539,7 +537,7 @@ __global__ void __launch_bounds__(kThreads, IPT == 16 ? 3 : 4) k_sweep(
         if (tid == 0) next = atomicAdd(counter, 1u);
 #pragma unroll
         for (int q = 0; q < VPT; ++q) {
-            const int bin = tid * VPT + q;
+            const int bin = tid + q * kThreads;
             if (bin >= BINS) continue;
             const uint32_t excl = look_back<BINS>(tile, status + bin, groups + bin, limit, err);
             if ((tile & (kGroup - 1)) == kGroup - 1)  // more than one tile
@@ -725,7 +723,7 @@ SortPlan make_sort_plan(int bits) {
     }
     // Up to 9-bit digits for short keys (tile ids); 7-bit digits for long keys
     // (depth): measured, four 7-bit passes over 27-bit depth keys beat three
-    // 9-bit ones (4.4 against 6.9 ps a key and pass: four times the counts to
+    // 9-bit ones (4.4 against 6.4 ps a key and pass: four times the counts to
     // publish and look back for, shorter runs, fewer CTAs per SM).
     // Keys wider than 28 bits (a far/near ratio beyond about 2^29) take four
     // wider digits: the scratch buffers hold at most kMaxSortPasses passes.
