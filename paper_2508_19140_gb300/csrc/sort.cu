@@ -338,6 +338,8 @@ __device__ __forceinline__ void carry_unpack(const RectCarry& rc, uint32_t k, ui
 // 217 -> 147 us (32 M keys, 7-bit digits; 3.6 TB/s moved), 36.6 -> 27 us (4 M
 // keys), 433 -> 322 us (62 M keys, 8-bit), 630 -> 493 us (77 M keys, 9-bit; a thread's
 // two bins 256 apart: 553 us with neighbouring ones, whose counters share banks).
+// Carrying the tile rects costs the 32 M depth passes 147 -> 163 us (sum 65 us) and
+// saves the duplication's random gather of them (0.33 -> 0.03 ms).
 template <int BITS, int IPT, int KIND>
 __global__ void __launch_bounds__(kThreads, IPT == 16 ? 3 : 4) k_sweep(
     const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint32_t* __restrict__ kout,
