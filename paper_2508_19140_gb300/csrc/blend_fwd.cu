@@ -295,15 +295,16 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_bilinear(
 
 // Gaussian: every warp owns an 8x4 sub-tile and goes through the tile's list
 // with no CTA-wide barrier. The records are staged once for all of the tile's
-// warps, in a ring of kFwdStages batches of kFwdBatch: one warp copies a batch
+// warps, in a ring of kFwdStages batches: one warp copies a batch
 // (cp.async) and the batch's mbarrier tells the others when it has landed; the
 // last warp to be done with a batch refills its slot with the batch kFwdStages
 // further on (whose point indices one of the warps has read meanwhile), so warps
 // may drift apart. Of every 32 records a warp ballots those whose box meets the
 // left and the right 4x4 half of its sub-tile, and each half composites its own
 // records, 16 lanes in lockstep, beside the other half's. A warp whose 32 pixels
-// have terminated only keeps count; once all of the tile's warps have, nothing
-// more is staged.
+// have terminated only keeps count, also of the rest of its batch (looked for
+// every 32 records: where splats of 50 pixels end the lists early, 288 -> 262
+// us); once all of the tile's warps have, nothing more is staged.
 // Bound by issue slots (86 % busy, about 15 instructions a record and warp).
 // Before, every warp gathered every record itself (three scattered 16-byte loads
 // a record and warp: the L1 pipe 70 % busy) and walked the records that met its
@@ -311,13 +312,20 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_bilinear(
 // Gaussians, BF16, 703 -> 566 us; 2 M at 1599x899 397 -> 311 us. Halves alone
 // were 660 and 356 us, the ring with batches of 32 records 611 and 357, of 64
 // 571 and 325 us, of 128 566 and 311 us.
-constexpr int kFwdBatch = 128;
+// The two warps of an 8x8 tile have shorter lists, and the ring is what limits
+// their CTAs on an SM: batches of 64 records. 2 M at 1599x899, C = 4, FP32: 128
+// records 332 us, 64 279 us, 32 283 us (every warp on its own 319 us); C = 16
+// 634, 376 and 342 us (510 us); 2 M at 4096x4096 1335, 1012 and 1024 us (1069 us);
+// 0.3 M at 1599x899, C = 4, 105, 104 and 114 us (133 us), C = 16 207, 126 and 138
+// us (173 us).
+template <int TS>
+constexpr int gauss_fwd_batch() { return TS == 8 ? 64 : 128; }
 constexpr int kFwdStages = 3;
 constexpr uint32_t kGaussStop = 2u;  // s_abort: every warp has finished
 
-template <int C, bool BF16>
+template <int TS, int C, bool BF16>
 constexpr size_t gauss_fwd_smem() {
-    return 128 + sizeof(uint32_t) * kFwdStages * kFwdBatch * gauss_ring_stride<C, BF16>();
+    return 128 + sizeof(uint32_t) * kFwdStages * gauss_fwd_batch<TS>() * gauss_ring_stride<C, BF16>();
 }
 
 template <int TS, int C, bool BF16>
@@ -329,7 +337,7 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_gauss(
     constexpr int NT = TS * TS;
     constexpr int NW = NT / 32;      // warps = 8x4 sub-tiles
     constexpr int WPR = TS / 8;      // warps per row of 8x4 sub-tiles
-    constexpr int GB = kFwdBatch;
+    constexpr int GB = gauss_fwd_batch<TS>();
     constexpr int R = kFwdStages;
     constexpr int NG = GB / 32;      // ballots per batch
     constexpr int RW = RecLayout<1, C, BF16>::words;
@@ -402,7 +410,7 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_gauss(
 #pragma unroll 1
     for (uint32_t j = 0; j < nb; ++j) {
         const int st = (int)(j % R);
-        const uint32_t fin = __ballot_sync(0xffffffffu, done);
+        uint32_t fin = __ballot_sync(0xffffffffu, done);
         if (fin == 0xffffffffu && !counted) {
             counted = true;
             if (lane == 0) atomicAdd(&s_fin, 1u);
@@ -475,6 +483,7 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_gauss(
                     }
                 }
             }
+            fin = __ballot_sync(0xffffffffu, done);
         }
         if (pref) {
 #pragma unroll
@@ -535,7 +544,7 @@ cudaError_t launch_fwd_t(const ViewTable& vt, const Bufs& b, const uint32_t* pts
         return launch_dependent(k_blend_fwd_bilinear<TS, RPT, C, BF16>, grid, TS * TS, smem, s, vt, b.ranges, b.order,
                                 pts, b.rec, b.rec_tile, b.t_final, b.last, b.hdr, b.trace);
     }
-    constexpr size_t smem = gauss_fwd_smem<C, BF16>();
+    constexpr size_t smem = gauss_fwd_smem<TS, C, BF16>();
     static_assert(smem <= 48 * 1024, "within the default dynamic shared memory");
     ProfScope ps("blend_fwd", s);
     return launch_dependent(k_blend_fwd_gauss<TS, C, BF16>, grid, TS * TS, smem, s, vt, b.ranges, b.order, pts, b.rec,
