@@ -761,12 +761,14 @@ __global__ void __launch_bounds__(TS * TS) k_blend_bwd_gauss(
 
 // The gradients of one point: its copies' rows in rect order, and for Gaussians
 // the chain rule to position and scale.
-template <int C, int MODE>
+// KNOWN: bit k of `replayed` says whether the backward blend reached copy k, for
+// a point with at most four copies (otherwise it is looked up here).
+template <int C, int MODE, bool KNOWN>
 __device__ __forceinline__ void reduce_point(const ViewTable& vt, const uint32_t* __restrict__ zbits,
                                              const uint2* __restrict__ rect, const uint32_t* __restrict__ rect4,
                                              const uint32_t* __restrict__ base, const uint2* __restrict__ cutoff,
                                              const float* __restrict__ partial, const float* __restrict__ grow,
-                                             int64_t gi) {
+                                             int64_t gi, uint32_t replayed) {
     constexpr int P = MODE == 0 ? C + 1 : C + 7;
     constexpr int PS = partial_stride(P);
     constexpr int GS = grow_stride(P);
@@ -797,7 +799,7 @@ __device__ __forceinline__ void reduce_point(const ViewTable& vt, const uint32_t
             return;
         }
     }
-    if (cnt && (MODE == 0 || cnt <= 4)) {
+    if (cnt && (MODE == 0 || (KNOWN && cnt <= 4))) {
         // At most four tiles (every bilinear point, nearly every small
         // Gaussian). The cutoffs of all of them first, then the rows (two at a
         // time for rows of up to 12 floats), so a point waits on two memory
@@ -807,8 +809,8 @@ __device__ __forceinline__ void reduce_point(const ViewTable& vt, const uint32_t
         bool dn[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            dn[k] = false;
-            if (k < (int)cnt) {
+            dn[k] = KNOWN && ((replayed >> k) & 1u);
+            if (!KNOWN && k < (int)cnt) {
                 const uint2 co = cutoff[V.tile_off + (int64_t)(ty0 + k / w) * V.tiles_x + (tx0 + k % w)];
                 dn[k] = zb < co.x || (zb == co.x && (uint32_t)gi <= co.y);
             }
@@ -948,7 +950,7 @@ __global__ void __launch_bounds__(256, 6) k_reduce_grads(const ViewTable vt, con
     dependency_sync(zbits, rect, rect4, base);
     const int64_t gi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (gi >= vt.n_total) return;
-    reduce_point<C, 0>(vt, zbits, rect, rect4, base, cutoff, partial, grow, gi);
+    reduce_point<C, 0, false>(vt, zbits, rect, rect4, base, cutoff, partial, grow, gi, 0u);
 }
 
 // Gaussian points. Behind the early termination of a dense frame most points
@@ -957,32 +959,68 @@ __global__ void __launch_bounds__(256, 6) k_reduce_grads(const ViewTable vt, con
 // others, scattered over all warps, are collected in shared memory and worked
 // on by full warps: every warp running the chain rule for a few of its lanes
 // took 546 us on that frame (46 % issue-active, 589 instructions a warp), this
-// 349 us. A point also counts as replayed where a factor of the chain may not
+// 335 us. A point also counts as replayed where a factor of the chain may not
 // be finite, so that its product with zero sums is not zero: a scale that is
 // not finite makes the rect cover the whole image, and a covariance may be
 // singular without dilation, or overflow next to the camera.
-template <int C>
-__global__ void __launch_bounds__(256, 4) k_reduce_gauss(const ViewTable vt, const uint32_t* __restrict__ zbits,
-                                                      const uint2* __restrict__ rect,
-                                                      const uint32_t* __restrict__ rect4,
-                                                      const uint32_t* __restrict__ base,
-                                                      const uint2* __restrict__ cutoff,
-                                                      const float* __restrict__ partial,
-                                                      const float* __restrict__ grow) {
-    dependency_sync(zbits, rect, rect4, base);
-    constexpr int K = 4;  // points per thread
-    __shared__ uint16_t s_queue[256 * K];
+// Bound by latency, so by the warps in flight. Where the backward blend replayed
+// more than about a copy a point, few points are left out and looking for them
+// costs a round trip and two barriers: there every thread takes its point. Times
+// taking every point / collecting (us, C = 4, 1599x899): 1.8 replayed copies a
+// point (2 M, 8x8 tiles) 105 / 128, 1.35 (3 M, 8x8) 141 / 156, 1.16 (4 M, 8x8)
+// 183 / 191, 1.0 (3 M, 16x16) 112 / 101, 0.77 (6 M, 8x8) 254 / 240, 0.29 (12 M,
+// 16x16) 373 / 251; 3.6 (splats of 50 pixels) 64 / 80. With wider rows the line lies
+// higher: 1.3 (2 M, 16x16) 80 / 80 for C = 4, 101 / 94 for C = 8, 146 / 129 for C =
+// 16; 1.8 (2 M, 8x8) 132 / 152 for C = 8, 194 / 214 for C = 16.
+// K: points a thread. Two for C = 16 where the points fill the GPU twice over all
+// the same (8 M points, 16x16 tiles: 351 -> 323 us; 2 M, 8x8: 193 -> 169 us; 60 k
+// points with 280 copies each 320 -> 374 us), one otherwise.
+template <int C, int K>
+__global__ void __launch_bounds__(256, C <= 8 ? 6 : 4) k_reduce_gauss(
+    const ViewTable vt, const uint32_t* __restrict__ zbits, const uint2* __restrict__ rect,
+    const uint32_t* __restrict__ rect4, const uint32_t* __restrict__ base, const uint2* __restrict__ cutoff,
+    const float* __restrict__ partial, const float* __restrict__ grow, const WsHeader* __restrict__ hdr) {
+    dependency_sync(zbits, rect, rect4, base, hdr);
+    const int64_t g0 = (int64_t)blockIdx.x * (256 * K);
+    if (8ull * hdr->needed_bwd > (unsigned long long)vt.n_total * (C <= 4 ? 9u : 12u)) {
+#pragma unroll 1
+        for (int k = 0; k < K; ++k) {
+            const int64_t gi = g0 + k * 256 + threadIdx.x;
+            if (gi < vt.n_total) reduce_point<C, 1, false>(vt, zbits, rect, rect4, base, cutoff, partial, grow, gi, 0u);
+        }
+        return;
+    }
+    __shared__ uint16_t s_queue[256 * K];  // point in the block | replayed ones of its first four copies << 12
     __shared__ uint32_t s_count;
     if (threadIdx.x == 0) s_count = 0;
     __syncthreads();
-    const int64_t g0 = (int64_t)blockIdx.x * (256 * K);
     uint2 rc[K];
-    uint32_t zb[K];
+    uint32_t zb[K], replayed[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) {
         const int64_t gi = g0 + k * 256 + threadIdx.x;
         rc[k] = gi < vt.n_total ? rect[gi] : make_uint2(1u, 0u);
         zb[k] = gi < vt.n_total ? zbits[gi] : 0u;
+    }
+    auto reached = [](uint2 co, uint32_t z, int64_t gi) { return z < co.x || (z == co.x && (uint32_t)gi <= co.y); };
+    // the first four tiles' cutoffs of the points in one round trip
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int64_t gi = g0 + k * 256 + threadIdx.x;
+        const int cnt = (int)rect_count(rc[k]);
+        replayed[k] = 0;
+        if (cnt == 0) continue;
+        const ViewDev& V = vt.v[view_of_point(vt, gi)];
+        const int tx0 = rc[k].x & 0xffff, w = (int)(rc[k].y & 0xffff) - tx0 + 1;
+        const uint2* row = cutoff + V.tile_off + (int64_t)(rc[k].x >> 16) * V.tiles_x + tx0;
+        uint2 co[4];
+#pragma unroll
+        for (int t = 0, dx = 0; t < 4; ++t) {
+            co[t] = t < cnt ? row[dx] : make_uint2(0u, 0u);
+            if (++dx == w) dx = 0, row += V.tiles_x;
+        }
+#pragma unroll
+        for (int t = 0; t < 4; ++t) replayed[k] |= t < cnt && reached(co[t], zb[k], gi) ? 1u << t : 0u;
     }
 #pragma unroll
     for (int k = 0; k < K; ++k) {
@@ -991,18 +1029,17 @@ __global__ void __launch_bounds__(256, 4) k_reduce_gauss(const ViewTable vt, con
         const ViewDev& V = vt.v[view_of_point(vt, gi)];
         const int tx0 = rc[k].x & 0xffff, ty0 = rc[k].x >> 16, tx1 = rc[k].y & 0xffff, ty1 = rc[k].y >> 16;
         const uint32_t cnt = rect_count(rc[k]);
-        bool hit = false;
-        if (cnt) {
-            hit = vt.dilation < 1e-6f || !(__uint_as_float(zb[k]) > 1e-5f) ||
-                  (rc[k].x == 0u && tx1 == V.tiles_x - 1 && ty1 == V.tiles_y - 1);
-            for (int ty = ty0; ty <= ty1 && !hit; ++ty)
-                for (int tx = tx0; tx <= tx1; ++tx) {
-                    const uint2 co = cutoff[V.tile_off + (int64_t)ty * V.tiles_x + tx];
-                    hit = hit || zb[k] < co.x || (zb[k] == co.x && (uint32_t)gi <= co.y);
-                }
+        bool work = replayed[k] != 0u;
+        if (cnt && !work) {
+            work = vt.dilation < 1e-6f || !(__uint_as_float(zb[k]) > 1e-5f) ||
+                   (rc[k].x == 0u && tx1 == V.tiles_x - 1 && ty1 == V.tiles_y - 1);
+            if (cnt > 4)
+                for (int ty = ty0; ty <= ty1 && !work; ++ty)
+                    for (int tx = tx0; tx <= tx1; ++tx)
+                        work = work || reached(cutoff[V.tile_off + (int64_t)ty * V.tiles_x + tx], zb[k], gi);
         }
-        if (hit) {
-            s_queue[atomicAdd(&s_count, 1u)] = (uint16_t)(k * 256 + threadIdx.x);
+        if (work) {
+            s_queue[atomicAdd(&s_count, 1u)] = (uint16_t)((k * 256 + threadIdx.x) | replayed[k] << 12);
             continue;
         }
         const int64_t i = gi - V.pt_off;
@@ -1020,8 +1057,13 @@ __global__ void __launch_bounds__(256, 4) k_reduce_gauss(const ViewTable vt, con
     }
     __syncthreads();
     const uint32_t n = s_count;
-    for (uint32_t q = threadIdx.x; q < n; q += 256)
-        reduce_point<C, 1>(vt, zbits, rect, rect4, base, cutoff, partial, grow, g0 + s_queue[q]);
+#pragma unroll 1
+    for (int k = 0; k < K; ++k) {
+        const uint32_t q = k * 256 + threadIdx.x;
+        if (q >= n) break;
+        const uint32_t e = s_queue[q];
+        reduce_point<C, 1, true>(vt, zbits, rect, rect4, base, cutoff, partial, grow, g0 + (e & 4095u), e >> 12);
+    }
 }
 
 template <int TS, int RPT, int C, bool BF16, bool TSRC>
@@ -1088,11 +1130,14 @@ cudaError_t launch_bwd_c(const ViewTable& vt, const Bufs& b, const uint32_t* pts
 
 template <int C>
 cudaError_t launch_reduce_c(const ViewTable& vt, const Bufs& b, cudaStream_t s) {
-    const int per = vt.mode == 0 ? 256 : 1024;  // points per block
-    const unsigned grid = (unsigned)((vt.n_total + per - 1) / per);
+    const auto blocks = [&](int per) { return (unsigned)((vt.n_total + per - 1) / per); };
     ProfScope ps("reduce_grads", s);
-    return launch_dependent(vt.mode == 0 ? k_reduce_grads<C> : k_reduce_gauss<C>, grid, 256, 0, s, vt, b.zbits, b.rect,
-                            b.rect4, b.base, b.cutoff, b.partial, b.grow);
+    if (vt.mode == 0)
+        return launch_dependent(k_reduce_grads<C>, blocks(256), 256, 0, s, vt, b.zbits, b.rect, b.rect4, b.base, b.cutoff,
+                                b.partial, b.grow);
+    const bool two = C > 8 && vt.n_total >= 512 * 1024;
+    return launch_dependent(two ? k_reduce_gauss<C, C <= 8 ? 1 : 2> : k_reduce_gauss<C, 1>, blocks(two ? 512 : 256), 256, 0, s,
+                            vt, b.zbits, b.rect, b.rect4, b.base, b.cutoff, b.partial, b.grow, b.hdr);
 }
 
 }  // namespace
