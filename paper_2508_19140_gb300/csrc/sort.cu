@@ -618,8 +618,12 @@ __global__ void __launch_bounds__(kThreads, IPT == 16 ? 3 : 4) k_sweep(
 // of 4096 keys, which spend the least on counts and look-back (4 M points 27.3
 // us a pass, with 1024-key tiles 42.3 us; 500 k points 10.8 against 12.8 us),
 // unless so few keys would occupy only a part of the SMs (20 k points 8.7
-// against 10.1 us, 60 k points 9.3 against 10.4 us).
-int sweep_ipt(int64_t expect) { return expect <= 256 * 1024 ? 4 : 16; }
+// against 10.1 us, 60 k points 9.3 against 10.4 us). Copies are counted on the
+// device and can be far more than expected (large Gaussians), up to the
+// capacity: small tiles only below 2 Mi, where they cost little if so (both
+// tile sort passes of 0.12 M Gaussians, small / large tiles: 0.2 M copies 34 / 38
+// us, 1.4 M 53 / 42 us, 4.4 M 119 / 73 us, 9.5 M 237 / 115 us).
+int sweep_ipt(int64_t expect, int64_t cap) { return expect <= 256 * 1024 && cap <= 2 * 1024 * 1024 ? 4 : 16; }
 
 template <int BITS, int IPT>
 cudaError_t sort_t(uint32_t* keys[2], uint32_t* vals[2], int64_t n, const uint32_t* d_n, int64_t cap, int64_t expect,
@@ -710,7 +714,7 @@ template <int BITS>
 cudaError_t sort_b(uint32_t* keys[2], uint32_t* vals[2], int64_t n, const uint32_t* d_n, int64_t cap, int64_t expect,
                    const SortPlan& plan, const SortScratch& sc, cudaStream_t s, int* result_buf,
                    const char* const names[2], bool identity_vals, bool keys_out, const CarryIo* carry) {
-    if (sweep_ipt(expect) == 4)
+    if (sweep_ipt(expect, cap) == 4)
         return sort_t<BITS, 4>(keys, vals, n, d_n, cap, expect, plan, sc, s, result_buf, names, identity_vals, keys_out, carry);
     return sort_t<BITS, 16>(keys, vals, n, d_n, cap, expect, plan, sc, s, result_buf, names, identity_vals, keys_out, carry);
 }
@@ -746,7 +750,7 @@ SortPlan make_sort_plan(int bits) {
 
 int64_t sort_status_words(const SortPlan& plan, int64_t cap, int64_t expect) {
     if (plan.passes == 0) return 0;
-    const StatusLayout l = status_layout<0>(cap, kThreads * sweep_ipt(expect));
+    const StatusLayout l = status_layout<0>(cap, kThreads * sweep_ipt(expect, cap));
     return plan.passes * (l.pass_words << plan.digit_bits[0]);
 }
 
