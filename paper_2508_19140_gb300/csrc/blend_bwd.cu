@@ -75,16 +75,29 @@ constexpr size_t bilinear_bwd_smem() {
            + 128;
 }
 
+// CTAs per SM the registers are held to. 8x8 tiles with one record per thread: as
+// many as shared memory lets an SM hold, 16 of up to 4 channels (64 registers),
+// fewer of wider records, which had spilled at 64: 4 M points, 1280x832, at 16 CTAs
+// / at these, C = 8: FP32 gather 306 / 306 us, record copy 269 / 262, BF16 275 / 266
+// and 249 / 227 us; C = 16: FP32 copy 596 / 541, BF16 561 / 507 and 520 / 441 us. The
+// C = 16 FP32 gather, bound by its scattered reads, is faster held to 64
+// registers all the same (875 us; 900 without spills).
+template <int TS, int RPT, int C, bool BF16, bool TSRC>
+constexpr int bilinear_bwd_ctas() {
+    if (TS != 8 || RPT != 1) return 1;
+    if (C <= 4) return 16;
+    if (C == 8) return BF16 ? 14 : 12;
+    return BF16 ? 11 : TSRC ? 8 : 16;
+}
+
 // RPT = records each thread stages per batch (blend depth D = TS * TS * RPT).
-// 8x8 tiles with one record per thread: held to 64 registers, so the 16 CTAs
-// per SM that shared memory allows stay resident (no spills at that bound).
 // TSRC: the workspace holds the forward's tile-ordered record copy, so each
 // batch is one contiguous run of records, staged by ONE TMA bulk copy
 // (cp.async.bulk, completed on a per-stage mbarrier) issued by thread 0; if
 // the last forward did not write the copy (header flag), the threads gather
 // the records by point index into the same ring instead.
 template <int TS, int RPT, int C, bool BF16, bool TSRC>
-__global__ void __launch_bounds__(TS * TS, TS == 8 && RPT == 1 ? 16 : 1) k_blend_bwd_bilinear(
+__global__ void __launch_bounds__(TS * TS, bilinear_bwd_ctas<TS, RPT, C, BF16, TSRC>()) k_blend_bwd_bilinear(
     const ViewTable vt, const uint2* __restrict__ ranges, const uint32_t* __restrict__ order,
     const uint32_t* __restrict__ pts, const uint32_t* __restrict__ rec, const uint32_t* __restrict__ rec_tile,
     const float* __restrict__ t_final, const uint32_t* __restrict__ last_in,
