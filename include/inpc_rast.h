@@ -92,8 +92,7 @@ typedef struct {
     float alpha_max;       /* alpha clamp (0.99) */
     float dilation;        /* screen-space dilation variance, Gaussian mode (0.16) */
     int32_t max_copies;    /* capacity: point-tile copies per point (0 = 4 bilinear, 16 Gaussian) */
-    int32_t flags;         /* 0 or an OR of RAST_FLAG_SAVE_FOR_BWD, RAST_FLAG_TEST_SORT_STALL and
-                              RAST_FLAG_TEST_BLEND_STALL */
+    int32_t flags;         /* 0 or an OR of RAST_FLAG_SAVE_FOR_BWD and the RAST_FLAG_TEST_* hooks */
 } rast_opts_t;
 
 /* The forward blend also writes a copy of every point record it reads, in
@@ -113,8 +112,8 @@ typedef struct {
  * runs out, the kernel sets the timeout bit of the workspace error word and
  * returns normally; every later stage sees the bit and produces an empty copy
  * list (images of zero coverage, zero point gradients), and
- * rasterize_get_status() returns RAST_ERR_TIMEOUT. Needs more than 4096
- * points. Never set outside tests. */
+ * rasterize_get_status() returns RAST_ERR_TIMEOUT. Needs more than one tile of
+ * keys (1024 for up to 256 Ki points, 4096 for more). Never set outside tests. */
 #define RAST_FLAG_TEST_SORT_STALL 1
 
 /* Test hook for the bounded waits of the Gaussian backward blend (failure
@@ -126,6 +125,23 @@ typedef struct {
  * normally (the point gradients are then incomplete), and
  * rasterize_get_status() returns RAST_ERR_TIMEOUT. Never set outside tests. */
 #define RAST_FLAG_TEST_BLEND_STALL 4
+
+/* The same for the Gaussian forward blend: the second batch (64 records on 8x8
+ * tiles, 128 on 16x16) of every tile that has one is never staged, and the
+ * waits on it are limited to 64 polls instead of 2^20. The images then hold
+ * what was blended before, and rasterize_get_status() returns
+ * RAST_ERR_TIMEOUT. Never set outside tests. */
+#define RAST_FLAG_TEST_FWD_BLEND_STALL 16
+
+/* Test hooks for the waits of the depth sort's first digit pass on the copies of
+ * a tile into shared memory: the keys (32) or the values (64) of its first tile
+ * are never copied, and the wait on them is limited to 64 polls instead of
+ * 2^20. As with RAST_FLAG_TEST_SORT_STALL nothing is blended and
+ * rasterize_get_status() returns RAST_ERR_TIMEOUT. The values are the points'
+ * tile rects, where these travel with the sort; elsewhere there are none to
+ * withhold. Never set outside tests. */
+#define RAST_FLAG_TEST_KEY_COPY_STALL 32
+#define RAST_FLAG_TEST_VALUE_COPY_STALL 64
 
 typedef struct {
     float* feat;    /* [H][W][C] out */

@@ -113,7 +113,9 @@ rast_status_t make_plan(const rast_view_t* views, int32_t n_views, const rast_op
     if (!untiled && !blend_depth_supported(o->mode, o->tile, depth)) return RAST_ERR_NOT_SUPPORTED;
     if (!(o->t_min >= 0.f) || !(o->alpha_max > 0.f && o->alpha_max < 1.f)) return RAST_ERR_ARG;
     if (!(o->dilation >= 0.f) || o->max_copies < 0) return RAST_ERR_ARG;
-    if ((o->flags & ~(RAST_FLAG_TEST_SORT_STALL | RAST_FLAG_SAVE_FOR_BWD | RAST_FLAG_TEST_BLEND_STALL)) != 0)
+    if ((o->flags & ~(RAST_FLAG_TEST_SORT_STALL | RAST_FLAG_SAVE_FOR_BWD | RAST_FLAG_TEST_BLEND_STALL |
+                      RAST_FLAG_TEST_FWD_BLEND_STALL | RAST_FLAG_TEST_KEY_COPY_STALL |
+                      RAST_FLAG_TEST_VALUE_COPY_STALL)) != 0)
         return RAST_ERR_ARG;
     const int C = views[0].pts.channels;
     const int dt = views[0].pts.feat_dtype;
@@ -461,6 +463,13 @@ namespace {
 const char* const kDepthSortNames[2] = {"depth_sort.hist", "depth_sort.sweep"};
 const char* const kTileSortNames[2] = {"tile_sort.hist", "tile_sort.sweep"};
 
+int sort_stall(int32_t flags) {
+    return flags & RAST_FLAG_TEST_SORT_STALL         ? kStallCounts
+           : flags & RAST_FLAG_TEST_KEY_COPY_STALL   ? kStallKeys
+           : flags & RAST_FLAG_TEST_VALUE_COPY_STALL ? kStallValues
+                                                     : kNoStall;
+}
+
 cudaError_t launch_init(const Plan& pl, const Bufs& b, cudaStream_t s) {
     const ViewTable& vt = pl.vt;
     ProfScope ps("init_header", s);
@@ -479,7 +488,7 @@ cudaError_t run_fwd(const Plan& pl, const Bufs& b, cudaStream_t s) {
         uint32_t* k[2] = {b.keyA[0], b.keyA[1]};
         uint32_t* v[2] = {b.valA[0], b.valA[1]};
         const SortScratch sc{b.sort_ghist, b.sort_counters, b.sort_status, &b.hdr->error,
-                             (vt.flags & RAST_FLAG_TEST_SORT_STALL) != 0};
+                             sort_stall(vt.flags)};
         const CarryIo io{pl.carry, vt.mode == 0 ? b.rect4 : b.valA[0], vt.mode == 1, b.rect, b.rectS};
         // Only the depth order of the point indices (and the points' rects in
         // that order) is used after this sort.
@@ -525,7 +534,7 @@ cudaError_t run_fwd_key64(const Plan& pl, const Bufs& b, cudaStream_t s) {
     RAST_TRY(launch_project(vt, b, false, RectCarry{}, s));
     RAST_TRY(launch_untiled_copies(vt, b, b.keyA[0], b.keyC[0], b.pixC, b.ptC, s));
     const SortScratch sc{b.sort_ghist, b.sort_counters, b.sort_status, &b.hdr->error,
-                         (vt.flags & RAST_FLAG_TEST_SORT_STALL) != 0};
+                         sort_stall(vt.flags)};
     static const char* const kLoNames[2] = {"sort64.lo.hist", "sort64.lo.sweep"};
     static const char* const kHiNames[2] = {"sort64.hi.hist", "sort64.hi.sweep"};
     int ra = 0, rb = 0;
@@ -542,7 +551,7 @@ cudaError_t run_fwd_key64(const Plan& pl, const Bufs& b, cudaStream_t s) {
         uint32_t* v[2] = {b.valC[g], b.valC[ra]};
         SortScratch sc2 = sc;
         sc2.ghist += kSortHistWords;
-        sc2.stall_test = false;
+        sc2.stall = kNoStall;
         RAST_TRY(radix_sort(k, v, 0, &b.hdr->n_copies, pl.copy_cap, pl.expectC, pl.planC, sc2, s, &rb, kHiNames));
     }
     const int r = key64_result_pair(pl);

@@ -102,10 +102,10 @@ __device__ __forceinline__ void bulk_copy_g2s(void* dst, const void* src, uint32
 }
 
 // Waits until the phase of `bar` with this parity has completed; false if it
-// did not within kMbarPolls polls.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
+// did not within `polls` polls.
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32_t polls = kMbarPolls) {
     const uint32_t b = smem_addr(bar);
-    for (uint32_t i = 0; i < kMbarPolls; ++i) {
+    for (uint32_t i = 0; i < polls; ++i) {
         uint32_t ok;
         asm volatile(
             "{\n\t.reg .pred p;\n\t"

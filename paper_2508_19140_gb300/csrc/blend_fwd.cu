@@ -387,7 +387,11 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_gauss(
 
     // Stages batch j (all 32 lanes of one warp). Batches j >= R take their point
     // indices from s_pnext.
+    // Test hook (RAST_FLAG_TEST_FWD_BLEND_STALL): batch 1 is never staged and the
+    // waits on it are short, so they run out.
+    const bool stall_test = (vt.flags & RAST_FLAG_TEST_FWD_BLEND_STALL) != 0;
     auto stage = [&](uint32_t j) {
+        if (stall_test && j == 1) return;
         const int st = (int)(j % R);
 #pragma unroll
         for (int k = 0; k < NG; ++k) {
@@ -415,7 +419,8 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_gauss(
             counted = true;
             if (lane == 0) atomicAdd(&s_fin, 1u);
         }
-        if (!__all_sync(0xffffffffu, mbar_wait_or_abort(&s_mbar[st], (phase >> st) & 1u, &s_abort, kMbarPolls))) {
+        const uint32_t polls = stall_test && j == 1 ? 64u : kMbarPolls;
+        if (!__all_sync(0xffffffffu, mbar_wait_or_abort(&s_mbar[st], (phase >> st) & 1u, &s_abort, polls))) {
             if (lane == 0 && *(volatile uint32_t*)&s_abort != kGaussStop) {
                 s_abort = 1u;
                 atomicOr(&hdr->error, kErrTimeout);

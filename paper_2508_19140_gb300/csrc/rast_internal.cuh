@@ -341,12 +341,15 @@ __device__ __forceinline__ uint32_t rect_code(const RectCarry& rc, uint32_t tx0,
     return tx0 | (ty0 << rc.tx_bits) | (w << (rc.tx_bits + rc.ty_bits)) | (h << (rc.tx_bits + rc.ty_bits + rc.span_bits));
 }
 
+// Test hooks of the sweeps' bounded waits: what the first tile withholds.
+enum SortStall { kNoStall = 0, kStallCounts = 1, kStallKeys = 2, kStallValues = 3 };
+
 struct SortScratch {
     uint32_t* ghist;     // [passes][bins], at most kSortHistWords, zeroed
     uint32_t* counters;  // [kMaxSortPasses]
     uint32_t* status;    // sort_status_words()
     uint32_t* err;       // workspace error word
-    bool stall_test = false;  // RAST_FLAG_TEST_SORT_STALL: the first pass's first tile never publishes
+    int stall = kNoStall;  // test hook, first pass
 };
 
 struct CarryIo {

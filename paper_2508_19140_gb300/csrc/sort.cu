@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(kThreads, IPT == 16 ? 3 : 4) k_sweep(
     const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint32_t* __restrict__ kout,
     uint32_t* __restrict__ vout, int64_t n_host, const uint32_t* d_n, int64_t cap, int shift,
     uint32_t mask, const uint32_t* __restrict__ ghist_pass, uint32_t* __restrict__ counter,
-    uint32_t* __restrict__ status, uint32_t* __restrict__ err, int stall_test, const CarryIo carry) {
+    uint32_t* __restrict__ status, uint32_t* __restrict__ err, int stall, const CarryIo carry) {
     dependency_sync(ghist_pass, err, d_n);
     constexpr bool IDV = KIND == kIdentity;
     constexpr int BINS = 1 << BITS;
@@ -387,8 +387,9 @@ __global__ void __launch_bounds__(kThreads, IPT == 16 ? 3 : 4) k_sweep(
         mbar_init_fence();
         s_tile = atomicAdd(counter, 1u);
         if (s_tile < ntiles) {
-            fetch(s_k, kin, s_tile, &s_mbar[0]);
-            if (!IDV) fetch(s_v, vin, s_tile, &s_mbar[1]);
+            // (test hooks: the first tile's keys or values never arrive)
+            if (stall != kStallKeys || s_tile != 0) fetch(s_k, kin, s_tile, &s_mbar[0]);
+            if (!IDV && (stall != kStallValues || s_tile != 0)) fetch(s_v, vin, s_tile, &s_mbar[1]);
         }
     }
     // Global start of every digit in this pass.
@@ -406,14 +407,16 @@ __global__ void __launch_bounds__(kThreads, IPT == 16 ? 3 : 4) k_sweep(
     __syncthreads();
     int64_t tile = s_tile;
     uint32_t phase = 0;
-    const uint32_t limit = stall_test ? 64u : (1u << 22);
+    const uint32_t limit = stall ? 64u : (1u << 22);
     while (tile < ntiles) {
         const int64_t base = tile * TILE;
         const int cnt = (int)(n - base < TILE ? n - base : TILE);
 #pragma unroll
         for (int i = 0; i < (BINS + 31) / 32; ++i)
             if (i * 32 + lane < BINS) tab[i * 32 + lane] = make_uint2(0u, 0u);
-        bool failed = !mbar_wait(&s_mbar[0], phase);
+        const uint32_t key_polls = stall == kStallKeys && tile == 0 ? 64u : kMbarPolls;
+        const uint32_t val_polls = stall == kStallValues && tile == 0 ? 64u : kMbarPolls;
+        bool failed = !mbar_wait(&s_mbar[0], phase, key_polls);
         // Keys past the end are all ones: they have the highest digit and come
         // last in input order, so they rank behind every real key.
         uint32_t k[IPT];
@@ -429,15 +432,15 @@ __global__ void __launch_bounds__(kThreads, IPT == 16 ? 3 : 4) k_sweep(
         for (int r = 0; r < IPT; ++r) atomicAdd(&tab[(k[r] >> shift) & mask].y, 1u);
         if (__syncthreads_or(failed)) {  // a copy never arrived: report it, let the other land, stop
             if (tid == 0) atomicOr(err, kErrTimeout);
-            mbar_wait(&s_mbar[0], phase);
+            mbar_wait(&s_mbar[0], phase, key_polls);
             if (!IDV) mbar_wait(&s_mbar[1], phase);
             break;
         }
 
-        // Publish the tile's counts (test hook: with stall_test the first tile
+        // Publish the tile's counts (test hook: with kStallCounts the first tile
         // publishes nothing, so its successor's wait runs out), and turn the
         // warps' counts into tile-local positions (digit, then warp).
-        const bool publish = ntiles > 1 && !(stall_test && tile == 0);
+        const bool publish = ntiles > 1 && !(stall == kStallCounts && tile == 0);
         uint32_t tot[VPT];           // the tile's count of this thread's bins, keys past the end left out
         uint32_t c[VPT][kWarps];     // each warp's count
         uint32_t local[VPT], inc[VPT];  // all of them, and their sums over the warp's lanes
@@ -482,10 +485,10 @@ __global__ void __launch_bounds__(kThreads, IPT == 16 ? 3 : 4) k_sweep(
                 }
             }
         }
-        if (!IDV) failed = !mbar_wait(&s_mbar[1], phase);
+        if (!IDV) failed = !mbar_wait(&s_mbar[1], phase, val_polls);
         if (__syncthreads_or(failed)) {
             if (tid == 0) atomicOr(err, kErrTimeout);
-            mbar_wait(&s_mbar[1], phase);
+            mbar_wait(&s_mbar[1], phase, val_polls);
             break;
         }
         phase ^= 1u;
@@ -702,7 +705,7 @@ cudaError_t sort_t(uint32_t* keys[2], uint32_t* vals[2], int64_t n, const uint32
         uint32_t* kout = (last && !keys_out) ? nullptr : keys[cur ^ 1];
         e = launch_dependent(kern, gs, kThreads, smem, s, keys[cur], vin, kout, vals[cur ^ 1], n, d_n, cap, shift, mask,
                              sc.ghist + k * BINS, sc.counters + k, sc.status + k * sl.pass_words, sc.err,
-                             (k == 0 && sc.stall_test) ? 1 : 0, carry ? *carry : CarryIo{});
+                             k == 0 ? sc.stall : (int)kNoStall, carry ? *carry : CarryIo{});
         if (e != cudaSuccess) return e;
         cur ^= 1;
     }

@@ -34,6 +34,9 @@ PASS_FWD, PASS_BWD = 1, 2
 FLAG_TEST_SORT_STALL = 1  # RAST_FLAG_TEST_SORT_STALL: failure-path tests only
 FLAG_SAVE_FOR_BWD = 2     # RAST_FLAG_SAVE_FOR_BWD: the forward keeps a tile-ordered record copy for the backward
 FLAG_TEST_BLEND_STALL = 4  # RAST_FLAG_TEST_BLEND_STALL: failure-path tests only
+FLAG_TEST_FWD_BLEND_STALL = 16  # the same for the Gaussian forward blend
+FLAG_TEST_KEY_COPY_STALL = 32  # and for the depth sort's copies of keys
+FLAG_TEST_VALUE_COPY_STALL = 64  # and of values
 
 
 class RastError(RuntimeError):
