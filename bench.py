@@ -183,10 +183,11 @@ def kernel_bytes(name, w):
         return 4 * (N if name.startswith("depth") else D)
     if name.endswith(".sweep"):     # per pass: read key+value, write key+value
         if name.startswith("depth"):
-            # the first pass reads the points' rects for the values it makes, the
-            # last writes them in place of the keys
+            # the first pass makes its values, from the points' rects where these
+            # travel with the sort; the last then writes the rects in place of the keys,
+            # or no keys
             passes = max(w.get("depth_passes", 1), 1)
-            return (16 * passes + rb - 4) * N / passes
+            return (16 * passes - 4 + (rb if w.get("carried", True) else -4)) * N / passes
         return 16 * D
     if name == "dup.count":   # rects in depth order (carried by the depth sort)
         return N * rb
@@ -196,6 +197,8 @@ def kernel_bytes(name, w):
         return N * (rb + 4) + D * 8
     if name == "ranges":      # a search of about 40 keys a tile
         return P * (8 + 4 * 40)
+    if name == "ranges.scan":  # large, sparsely covered images: every key, the ranges' ends
+        return D * 4 + P * 8
     if name == "blend_fwd":
         return Dn * (rec + 4) + P * 8 + HW * (4 * C + 16)
     if name == "point_slots":
@@ -438,7 +441,7 @@ def run_ours(args, ws_, rank, local):
              needed_bwd=int(stats["needed_records_bwd"]),
              HW=sum(v.camera.width * v.camera.height for v in scene.views), C=C,
              P=int(stats["n_tiles"]), rec_bytes=rec_bytes, feat_bytes=2 if bf16 else 4,
-             partial_floats=C + (7 if gauss else 1), gauss=gauss,
+             partial_floats=C + (7 if gauss else 1), gauss=gauss, carried="dup.gather" not in prof,
              depth_passes=int(round(prof.get("depth_sort.sweep", (0, 0))[0] / max(prof.get("init_header", (1, 0))[0], 1))))
     peak, peak_src = measured_peak_hbm()
     kernels = {}

@@ -252,8 +252,9 @@ rast_status_t make_plan(const rast_view_t* views, int32_t n_views, const rast_op
     pl.planA = make_sort_plan(bit_length(key_max));
     pl.planC = make_sort_plan(bit_length((uint64_t)(ntile > 0 ? ntile - 1 : 0)));
     // The rects travel with the depth sort when their code fits beside key and
-    // index (any usual frame: 27-bit keys, up to 32 M points, 1920x1080 at 8x8
-    // tiles); else the duplication gathers them in depth order.
+    // index (any usual frame, with 27-bit keys: up to 32 M bilinear points on
+    // 1920x1080 at 8x8 tiles; up to 16 M Gaussians there, 32 M at 16x16); else the
+    // duplication gathers them in depth order.
     {
         int tx = 0, ty = 0;
         for (int k = 0; k < n_views; ++k) {

@@ -591,7 +591,7 @@ cudaError_t launch_duplicate(const ViewTable& vt, const Bufs& b, const uint32_t*
     const int64_t nb = (n + kScanItems - 1) / kScanItems;
     if (nb == 0) return cudaSuccess;  // the header was zeroed at the start of the pass
     {
-        ProfScope ps("dup.count", s);
+        ProfScope ps(carried ? "dup.count" : "dup.gather", s);
         auto kern = vt.mode == 0 ? (carried ? k_dup_count<true, true> : k_dup_count<true, false>)
                                  : (carried ? k_dup_count<false, true> : k_dup_count<false, false>);
         const void* in = vt.mode == 0 ? (const void*)b.rect4 : (const void*)b.rect;
@@ -649,7 +649,7 @@ cudaError_t launch_ranges(const ViewTable& vt, const Bufs& b, const uint32_t* so
         int64_t g = (b.copy_cap + kT - 1) / kT;
         const int64_t gmax = (int64_t)device_sm_count() * 8;
         if (g > gmax) g = gmax;
-        ProfScope ps("ranges", s);
+        ProfScope ps("ranges.scan", s);
         k_ranges<<<(unsigned)g, kT, 0, s>>>(sorted_tiles, b.hdr, b.ranges);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
