@@ -39,13 +39,13 @@ int bit_length(uint64_t x) {
 
 enum Slot {
     S_HDR, S_REC, S_RECT, S_CNT, S_ZBITS, S_KEYA0, S_KEYA1, S_VALA0, S_VALA1, S_RECTS, S_BASE, S_BLK,
-    S_KEYC0, S_KEYC1, S_VALC0, S_VALC1, S_PARTIAL, S_GROW, S_SGHIST, S_SCOUNT, S_SSTATUS, S_RANGES, S_ORDER, S_CUTOFF, S_TRACE,
+    S_KEYC0, S_KEYC1, S_VALC0, S_VALC1, S_PARTIAL, S_GROW, S_SGHIST, S_SCOUNT, S_RANGES, S_ORDER, S_CUTOFF, S_TRACE,
     S_TFINAL, S_LAST, S_PIXC, S_PTC, S_RECTILE, S_COUNT
 };
 const char* kSlotNames[S_COUNT] = {
     "header", "records", "rect", "count", "zbits", "keys_a0", "keys_a1", "vals_a0", "vals_a1",
     "rect_sorted", "base", "block_sums", "keys_c0", "keys_c1", "vals_c0", "vals_c1",
-    "partial", "grad_rows", "sort_hist", "sort_counters", "sort_status", "ranges", "tile_order", "cutoff", "tile_trace", "t_final", "last",
+    "partial", "grad_rows", "sort_hist", "sort_counters", "ranges", "tile_order", "cutoff", "tile_trace", "t_final", "last",
     "copy_pixel", "copy_point", "records_tiled"};
 
 // Arrangements of the pipeline.
@@ -60,6 +60,7 @@ struct Plan {
     size_t off[S_COUNT];
     size_t bytes[S_COUNT];
     size_t total;
+    size_t status_bytes;  // the sorts' look-back words, in S_PARTIAL
     int64_t copy_cap, blk_cap;
     int64_t expectA, expectC;  // elements the two sorts are expected to have (their launch shapes)
     SortPlan planA, planC;
@@ -303,8 +304,8 @@ rast_status_t make_plan(const rast_view_t* views, int32_t n_views, const rast_op
     }
     // The sorts' look-back words live where the backward's partial rows will
     // (no sort runs in a backward pass, no partial row outlives one).
-    pl.bytes[S_SSTATUS] = 0;
-    if (pl.bytes[S_PARTIAL] < (size_t)sort_words * 4) pl.bytes[S_PARTIAL] = (size_t)sort_words * 4;
+    pl.status_bytes = (size_t)sort_words * 4;
+    if (pl.bytes[S_PARTIAL] < pl.status_bytes) pl.bytes[S_PARTIAL] = pl.status_bytes;
     pl.bytes[S_PIXC] = pl.bytes[S_PTC] = arrangement == kUntiledKey64 ? (size_t)D * 4 : 0;
     // Bilinear tiled: the forward blend writes every record it reads, in
     // tile-list order, so the backward reads its batches sequentially.
@@ -642,15 +643,18 @@ int32_t rasterize_workspace_layout(const rast_view_t* views, int32_t n_views, co
 namespace rast {
 namespace {
 
-// Every workspace array as (name, offset, bytes), then the aliases of the
-// sort results: "depth_sorted" (point indices in depth order), "sorted_keys"
-// and "sorted_vals" (the slots given).
+// Every workspace array as (name, offset, bytes), then the aliases: the sort
+// results "depth_sorted" (point indices in depth order), "sorted_keys" and
+// "sorted_vals" (the slots given), and "sort_status", the look-back words of the
+// call's last sort (the backward's partial rows lie over them).
 int32_t write_layout(const Plan& pl, int keys_slot, int vals_slot, rast_ws_entry_t* out, int32_t max) {
     const int ra = pl.planA.passes & 1;
-    struct Alias { const char* name; int slot; };
-    const Alias extra[] = {{"depth_sorted", ra ? S_VALA1 : S_VALA0},
-                           {"sorted_keys", keys_slot},
-                           {"sorted_vals", vals_slot}};
+    struct Alias { const char* name; int slot; size_t bytes; };
+    const int depth_slot = ra ? S_VALA1 : S_VALA0;
+    const Alias extra[] = {{"depth_sorted", depth_slot, pl.bytes[depth_slot]},
+                           {"sorted_keys", keys_slot, pl.bytes[keys_slot]},
+                           {"sorted_vals", vals_slot, pl.bytes[vals_slot]},
+                           {"sort_status", S_PARTIAL, pl.status_bytes}};
     int n = 0;
     for (int k = 0; k < S_COUNT; ++k, ++n) {
         if (out && n < max) {
@@ -663,7 +667,7 @@ int32_t write_layout(const Plan& pl, int keys_slot, int vals_slot, rast_ws_entry
         if (out && n < max) {
             std::snprintf(out[n].name, sizeof(out[n].name), "%s", a.name);
             out[n].offset = (int64_t)pl.off[a.slot];
-            out[n].bytes = (int64_t)pl.bytes[a.slot];
+            out[n].bytes = (int64_t)a.bytes;
         }
         ++n;
     }

@@ -303,13 +303,6 @@ __device__ __forceinline__ BilinGeom bilin_geom(float u, float v) {
     return g;
 }
 
-// Bilinear weight of the fragment at pixel (px, py) (a pixel of the 2x2 box).
-__device__ __forceinline__ float bilin_weight(int px, int py, int i0, int j0, float a, float b) {
-    const float wx = (px == i0) ? __fsub_rn(1.f, a) : a;
-    const float wy = (py == j0) ? __fsub_rn(1.f, b) : b;
-    return __fmul_rn(wx, wy);
-}
-
 // Gaussian pixel box from the record's radius r (inclusive, unclipped).
 struct GaussBox {
     int x0, x1, y0, y1;

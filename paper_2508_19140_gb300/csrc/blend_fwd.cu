@@ -188,9 +188,9 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_bilinear(
         for (int k = 0; k < RPT; ++k) {
             const int r = k * NT + tid;
             if (rel0 + r < len) {
-                // Per record: the four fragment alphas of its 2x2 box (the ops of
-                // bilin_weight and the clamp, so every pixel sees the same FP32
-                // bits) and one mask bit per covered pixel of this tile.
+                // Per record: the four fragment alphas of its 2x2 box (weights and
+                // clamp in rounded operations, the same FP32 bits for every pixel)
+                // and one mask bit per covered pixel of this tile.
                 const uint4 g = *reinterpret_cast<const uint4*>(ring + r * RS);
                 if (rec_tile) {
                     // The record, in list order, for the backward's sequential reads

@@ -156,14 +156,13 @@ __device__ __forceinline__ void load_counts(const uint32_t* __restrict__ p, int6
     }
 }
 
-template <bool P4>
-__global__ void __launch_bounds__(kT) k_count_blocks(const uint32_t* __restrict__ cnt, int64_t n,
+// The untiled baseline's copies a block and, with them scanned, a point's first copy.
+__global__ void __launch_bounds__(kT) k_count_blocks(const uint32_t* __restrict__ rect4, int64_t n,
                                                      uint32_t* __restrict__ blk) {
-    dependency_sync(cnt);
     __shared__ uint32_t s_warp[33];
     const int64_t s0 = (int64_t)blockIdx.x * kScanItems + (int64_t)threadIdx.x * kPer;
     uint32_t v[kPer];
-    load_counts<P4>(cnt, s0, n, v);
+    load_counts<true>(rect4, s0, n, v);
     uint32_t sum = 0;
 #pragma unroll
     for (int j = 0; j < kPer; ++j) sum += v[j];
@@ -194,7 +193,7 @@ __global__ void __launch_bounds__(1024) k_scan_blocks(uint32_t* __restrict__ blk
         blk[t] = run;
         run += c;
     }
-    if (hdr && threadIdx.x == 0) {
+    if (threadIdx.x == 0) {
         unsigned long long total = 0;
         for (int w = 0; w < 32; ++w) total += s_wtot[w];
         const bool over = total > (unsigned long long)cap;
@@ -329,15 +328,13 @@ __global__ void __launch_bounds__(kTW) k_dup_write(const ViewTable vt, const uin
     }
 }
 
-template <bool P4>
-__global__ void __launch_bounds__(kT) k_scan_apply(const uint32_t* __restrict__ cnt, int64_t n,
+__global__ void __launch_bounds__(kT) k_scan_apply(const uint32_t* __restrict__ rect4, int64_t n,
                                                    const uint32_t* __restrict__ blk,
                                                    uint32_t* __restrict__ base) {
-    dependency_sync(cnt, blk);
     __shared__ uint32_t s_warp[33];
     const int64_t s0 = (int64_t)blockIdx.x * kScanItems + (int64_t)threadIdx.x * kPer;
     uint32_t v[kPer];
-    load_counts<P4>(cnt, s0, n, v);
+    load_counts<true>(rect4, s0, n, v);
     uint32_t sum = 0;
 #pragma unroll
     for (int j = 0; j < kPer; ++j) sum += v[j];
@@ -559,12 +556,12 @@ cudaError_t launch_untiled_copies(const ViewTable& vt, const Bufs& b, const uint
     if (nb == 0) return cudaSuccess;
     {
         ProfScope ps("dup.count", s);
-        k_count_blocks<true><<<(unsigned)nb, kT, 0, s>>>(b.rect4, n, b.blk);
+        k_count_blocks<<<(unsigned)nb, kT, 0, s>>>(b.rect4, n, b.blk);
     }
     {
         ProfScope ps("dup.scan", s);
         k_scan_blocks<<<1, 1024, 0, s>>>(b.blk, nb, b.hdr, b.copy_cap);
-        k_scan_apply<true><<<(unsigned)nb, kT, 0, s>>>(b.rect4, n, b.blk, b.base);
+        k_scan_apply<<<(unsigned)nb, kT, 0, s>>>(b.rect4, n, b.blk, b.base);
     }
     {
         ProfScope ps("dup.write", s);
