@@ -126,11 +126,11 @@ typedef struct {
  * rasterize_get_status() returns RAST_ERR_TIMEOUT. Never set outside tests. */
 #define RAST_FLAG_TEST_BLEND_STALL 4
 
-/* The same for the Gaussian forward blend: the second batch (64 records on 8x8
- * tiles, 128 on 16x16) of every tile that has one is never staged, and the
- * waits on it are limited to 64 polls instead of 2^20. The images then hold
- * what was blended before, and rasterize_get_status() returns
- * RAST_ERR_TIMEOUT. Never set outside tests. */
+/* The same for the Gaussian forward blend of four FP32 channels: the second batch
+ * of 128 records (64 on large images at 8x8 tiles) of every tile that has one
+ * is never staged, and the waits on the batches are limited to 64 polls instead
+ * of 2^20. The images then hold what was blended before, and
+ * rasterize_get_status() returns RAST_ERR_TIMEOUT. Never set outside tests. */
 #define RAST_FLAG_TEST_FWD_BLEND_STALL 16
 
 /* Test hooks for the waits of the depth sort's first digit pass on the copies of

@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_bilinear(
 // may drift apart. Of every 32 records a warp ballots those whose box meets the
 // left and the right 4x4 half of its sub-tile, and each half composites its own
 // records, 16 lanes in lockstep, beside the other half's. A warp whose 32 pixels
-// have terminated only keeps count, also of the rest of its batch (looked for
+// have terminated only keeps count, also of the rest of its batch (looked at
 // every 32 records: where splats of 50 pixels end the lists early, 288 -> 262
 // us); once all of the tile's warps have, nothing more is staged.
 // Bound by issue slots (86 % busy, about 15 instructions a record and warp).
@@ -312,23 +312,27 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_bilinear(
 // Gaussians, BF16, 703 -> 566 us; 2 M at 1599x899 397 -> 311 us. Halves alone
 // were 660 and 356 us, the ring with batches of 32 records 611 and 357, of 64
 // 571 and 325 us, of 128 566 and 311 us.
-// The two warps of an 8x8 tile have shorter lists, and the ring is what limits
-// their CTAs on an SM: batches of 64 records. 2 M at 1599x899, C = 4, FP32: 128
-// records 332 us, 64 279 us, 32 283 us (every warp on its own 319 us); C = 16
-// 634, 376 and 342 us (510 us); 2 M at 4096x4096 1335, 1012 and 1024 us (1069 us);
-// 0.3 M at 1599x899, C = 4, 105, 104 and 114 us (133 us), C = 16 207, 126 and 138
-// us (173 us).
-template <int TS>
-constexpr int gauss_fwd_batch() { return TS == 8 ? 64 : 128; }
+// On 8x8 tiles the ring of 128 records, shared by two warps, is what limits the
+// CTAs on an SM. Where tiles are many times what fits, CTAs count more than long
+// batches, and a batch has 64 records; up to ten times what fits with 128, the
+// longest lists count, and it has 128. 1599x899 (22600 tiles, 13 times), 2 M, FP32:
+// C = 4 332 us with 128, 279 with 64, 283 with 32 (every warp on its own 319 us),
+// C = 16 634, 376, 342 us (510 us); 1200x720 (8 times), C = 4, 0.26 M / 1.2 M / 4.3 M
+// Gaussians: 103 / 209 / 296 us with 128, 117 / 214 / 272 us with 64; 660x396 (2.5
+// times): 69 / 184 / 250 and 72 / 201 / 271 us.
 constexpr int kFwdStages = 3;
+constexpr int kFwdBatch = 128, kFwdShortBatch = 64;
 constexpr uint32_t kGaussStop = 2u;  // s_abort: every warp has finished
 
-template <int TS, int C, bool BF16>
+template <int GB, int C, bool BF16>
 constexpr size_t gauss_fwd_smem() {
-    return 128 + sizeof(uint32_t) * kFwdStages * gauss_fwd_batch<TS>() * gauss_ring_stride<C, BF16>();
+    return 128 + sizeof(uint32_t) * kFwdStages * GB * gauss_ring_stride<C, BF16>();
 }
 
-template <int TS, int C, bool BF16>
+// GB: records per batch. STALL: test hook, batch 1 is never staged and the waits
+// are short, so those on it run out (a kernel of its own: a limit that is not a
+// constant cost the 8-channel blends 4 %).
+template <int TS, int GB, int C, bool BF16, bool STALL>
 __global__ void __launch_bounds__(TS * TS) k_blend_fwd_gauss(
     const ViewTable vt, const uint2* __restrict__ ranges, const uint32_t* __restrict__ order,
     const uint32_t* __restrict__ pts, const uint32_t* __restrict__ rec, float* __restrict__ t_final,
@@ -337,7 +341,6 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_gauss(
     constexpr int NT = TS * TS;
     constexpr int NW = NT / 32;      // warps = 8x4 sub-tiles
     constexpr int WPR = TS / 8;      // warps per row of 8x4 sub-tiles
-    constexpr int GB = gauss_fwd_batch<TS>();
     constexpr int R = kFwdStages;
     constexpr int NG = GB / 32;      // ballots per batch
     constexpr int RW = RecLayout<1, C, BF16>::words;
@@ -387,11 +390,8 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_gauss(
 
     // Stages batch j (all 32 lanes of one warp). Batches j >= R take their point
     // indices from s_pnext.
-    // Test hook (RAST_FLAG_TEST_FWD_BLEND_STALL): batch 1 is never staged and the
-    // waits on it are short, so they run out.
-    const bool stall_test = (vt.flags & RAST_FLAG_TEST_FWD_BLEND_STALL) != 0;
     auto stage = [&](uint32_t j) {
-        if (stall_test && j == 1) return;
+        if (STALL && j == 1) return;
         const int st = (int)(j % R);
 #pragma unroll
         for (int k = 0; k < NG; ++k) {
@@ -414,13 +414,12 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_gauss(
 #pragma unroll 1
     for (uint32_t j = 0; j < nb; ++j) {
         const int st = (int)(j % R);
-        uint32_t fin = __ballot_sync(0xffffffffu, done);
+        const uint32_t fin = __ballot_sync(0xffffffffu, done);
         if (fin == 0xffffffffu && !counted) {
             counted = true;
             if (lane == 0) atomicAdd(&s_fin, 1u);
         }
-        const uint32_t polls = stall_test && j == 1 ? 64u : kMbarPolls;
-        if (!__all_sync(0xffffffffu, mbar_wait_or_abort(&s_mbar[st], (phase >> st) & 1u, &s_abort, polls))) {
+        if (!__all_sync(0xffffffffu, mbar_wait_or_abort(&s_mbar[st], (phase >> st) & 1u, &s_abort, STALL ? 64u : kMbarPolls))) {
             if (lane == 0 && *(volatile uint32_t*)&s_abort != kGaussStop) {
                 s_abort = 1u;
                 atomicOr(&hdr->error, kErrTimeout);
@@ -488,7 +487,7 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_gauss(
                     }
                 }
             }
-            fin = __ballot_sync(0xffffffffu, done);
+            if (__all_sync(0xffffffffu, done)) break;
         }
         if (pref) {
 #pragma unroll
@@ -534,6 +533,24 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_gauss(
         atomicAdd(&hdr->needed, (unsigned long long)(open ? (rg.y - rg.x) : s_maxstop));
 }
 
+template <int TS, int C, bool BF16>
+cudaError_t launch_fwd_gauss(const ViewTable& vt, const Bufs& b, const uint32_t* pts, cudaStream_t s) {
+    constexpr size_t smem = gauss_fwd_smem<kFwdBatch, C, BF16>(), small = gauss_fwd_smem<kFwdShortBatch, C, BF16>();
+    static_assert(smem <= 48 * 1024, "within the default dynamic shared memory");
+    constexpr int64_t per_sm = 227 * 1024 / (smem + 3 * 1024);  // CTAs on an SM, with the static and the system's share
+    const unsigned grid = (unsigned)vt.tiles_total;
+    const bool short_batch = TS == 8 && vt.tiles_total > 10 * per_sm * device_sm_count();
+    constexpr int GS = TS == 8 ? kFwdShortBatch : kFwdBatch;
+    auto kern = short_batch ? k_blend_fwd_gauss<TS, GS, C, BF16, false> : k_blend_fwd_gauss<TS, kFwdBatch, C, BF16, false>;
+    if constexpr (C == 4 && !BF16) {
+        if (vt.flags & RAST_FLAG_TEST_FWD_BLEND_STALL)
+            kern = short_batch ? k_blend_fwd_gauss<TS, GS, C, BF16, true> : k_blend_fwd_gauss<TS, kFwdBatch, C, BF16, true>;
+    }
+    ProfScope ps("blend_fwd", s);
+    return launch_dependent(kern, grid, TS * TS, short_batch ? small : smem, s, vt, b.ranges, b.order, pts, b.rec, b.t_final,
+                            b.last, b.hdr);
+}
+
 template <int TS, int RPT, int C, bool BF16>
 cudaError_t launch_fwd_t(const ViewTable& vt, const Bufs& b, const uint32_t* pts, cudaStream_t s) {
     const unsigned grid = (unsigned)vt.tiles_total;
@@ -549,11 +566,7 @@ cudaError_t launch_fwd_t(const ViewTable& vt, const Bufs& b, const uint32_t* pts
         return launch_dependent(k_blend_fwd_bilinear<TS, RPT, C, BF16>, grid, TS * TS, smem, s, vt, b.ranges, b.order,
                                 pts, b.rec, b.rec_tile, b.t_final, b.last, b.hdr, b.trace);
     }
-    constexpr size_t smem = gauss_fwd_smem<TS, C, BF16>();
-    static_assert(smem <= 48 * 1024, "within the default dynamic shared memory");
-    ProfScope ps("blend_fwd", s);
-    return launch_dependent(k_blend_fwd_gauss<TS, C, BF16>, grid, TS * TS, smem, s, vt, b.ranges, b.order, pts, b.rec,
-                            b.t_final, b.last, b.hdr);
+    return launch_fwd_gauss<TS, C, BF16>(vt, b, pts, s);
 }
 
 template <int TS, int C, bool BF16>

@@ -124,3 +124,20 @@ def test_singular_covariance_without_dilation():
         g = r.grads()
         assert np.all(g["d_feat"][:2] == 0) and np.all(g["d_opacity"][:2] == 0)
         assert np.all(np.isnan(g["d_xyz"][:2])) and np.all(np.isnan(g["d_scale"][:2]))
+
+
+@pytest.mark.parametrize("tile", [8, 16])
+@pytest.mark.parametrize("n", [1, 31, 63, 64, 65, 127, 128, 129, 192, 193, 384, 385, 513])
+def test_gradients_of_short_lists(n, tile):
+    """Lists at the edges of the blends' batches, with a gradient comparison that no near pixel skips."""
+    v = _view(n, 8, 8, n)
+    kw = dict(mode="gaussian", gauss_cov="ewa", tile=tile, pin32=True)
+    keep = _keep(v, kw)
+    assert 2 * keep.sum() >= n
+    r = Run([v], mode="gaussian", tile=tile, backward=True)
+    assert r.status == 0
+    ref = oracle.backward(v.xyz, v.opacity, v.feat, v.camera, v.g_feat, v.g_alpha, v.g_depth, scale=v.scale, **kw)
+    g = r.grads()
+    _check_grad(g["d_feat"], ref["d_feat"], mask=keep)
+    for k in ("d_opacity", "d_xyz", "d_scale"):
+        _check_grad(g[k], ref[k], norm=1e-4, er=1e-3, ea=1e-5, mask=keep)
