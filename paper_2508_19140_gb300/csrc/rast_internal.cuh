@@ -175,12 +175,13 @@ __device__ __forceinline__ uint32_t rect_count(uint2 r) {
 // the one before it wrote. Launched this way a kernel is set up on the device
 // while the one before it drains, and dependency_sync, the first thing every
 // thread of such a kernel does, waits until that one is complete and its writes
-// are visible. 20 k points, 13 kernels: 130.5 -> 104.5 us a call; 4 M points,
-// forward and backward, 18 kernels: 739 -> 693 us; 62 M: 10.09 -> 10.04 ms. No
+// are visible. 20 k points, 15 kernels: 130.5 -> 104.5 us a call; 4 M points,
+// forward and backward, 20 kernels: 739 -> 693 us; 62 M: 10.09 -> 10.04 ms. No
 // kernel releases the next one early (launch_dependents): its blocks would sit
 // on SMs that the running kernel's last blocks could use (785 us and 11.17 ms).
-// The first kernel of a call is launched in the ordinary way, after everything
-// before it.
+// The first kernel of a pass (k_init, k_bwd_init) is launched in the ordinary way,
+// after everything before it, and so are the scan for the tile ranges with the
+// bucket count after it, and the untiled baselines' own kernels.
 // The __restrict__ pointers from which a kernel's first loads come go through
 // dependency_sync: a load through such a parameter counts as unaffected by
 // anything but the kernel's own accesses through it and could be moved above
