@@ -157,15 +157,15 @@ def measured_peak_hbm():
 # gradient-row scatters move 64-byte DRAM bursts, hence traffic above the
 # algorithmic bytes (profiles/ncu_blend_traffic_all_workloads.md).
 MEASURED_TRAFFIC = {
-    ("blend_fwd", 2, 8, 64, 0): 321559040,
-    ("blend_bwd", 2, 8, 64, 0): 705297664,
-    ("blend_fwd", 2, 8, 64, 1): 527894784,
-    ("blend_bwd", 2, 8, 64, 1): 409280000,
-    ("blend_fwd", 3, 16, 256, 0): 2889582080,
-    ("blend_fwd", 4, 16, 256, 0): 454670848,
-    ("blend_bwd", 4, 16, 256, 0): 1148037632,
-    ("blend_fwd", 5, 8, 64, 1): 9697941760,
-    ("blend_bwd", 5, 8, 64, 1): 9251388928,
+    ("blend_fwd", 2, 8, 64, 0): 321854720,
+    ("blend_bwd", 2, 8, 64, 0): 705271552,
+    ("blend_fwd", 2, 8, 64, 1): 528494336,
+    ("blend_bwd", 2, 8, 64, 1): 409503488,
+    ("blend_fwd", 3, 16, 256, 0): 2886308096,
+    ("blend_fwd", 4, 16, 256, 0): 454840832,
+    ("blend_bwd", 4, 16, 256, 0): 1149494528,
+    ("blend_fwd", 5, 8, 64, 1): 9702736896,
+    ("blend_bwd", 5, 8, 64, 1): 9161312000,
 }
 
 def kernel_bytes(name, w):

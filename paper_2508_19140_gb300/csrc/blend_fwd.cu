@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(TS * TS) k_blend_fwd_bilinear(
 // have terminated only keeps count, also of the rest of its batch (looked at
 // every 32 records: where splats of 50 pixels end the lists early, 288 -> 262
 // us); once all of the tile's warps have, nothing more is staged.
-// Bound by issue slots (86 % busy, about 15 instructions a record and warp).
+// Bound by issue slots (90 % busy, about 15 instructions a record and warp).
 // Before, every warp gathered every record itself (three scattered 16-byte loads
 // a record and warp: the L1 pipe 70 % busy) and walked the records that met its
 // whole sub-tile (of 32 records with 3-pixel boxes about 9; a half meets 6): 16 M

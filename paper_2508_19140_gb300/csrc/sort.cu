@@ -328,8 +328,8 @@ __device__ __forceinline__ void carry_unpack(const RectCarry& rc, uint32_t k, ui
 // buffer while this tile is written out, and its values into the spare one
 // after that. No thread holds values or waits on a global load.
 //
-// Bound by the shared-memory pipe (about one wavefront a key: counting, ranking
-// and scattering by digit; 75 % of its cycles on 32 M keys), then by the integer
+// Bound by the L1 data pipe (about one shared-memory wavefront a key: counting,
+// ranking and scattering by digit; 74 % of its cycles on 8 M keys), then by the integer
 // pipe. The ranking takes the lane masks of every other round from ballots
 // (integer pipe) and of the rounds between from a shared atomic OR (memory
 // pipe): all rounds from ballots were 172 us, all from the OR 159 us, both in
