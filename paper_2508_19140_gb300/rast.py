@@ -470,7 +470,7 @@ class _Batch(torch.autograd.Function):
             opts_kw = dict(opts_kw, flags=int(opts_kw.get("flags", 0)) | FLAG_SAVE_FOR_BWD)
         opts = make_opts(**opts_kw)
         dev = flat[0].device
-        pts, views, outs = [], [], []
+        pts, views, outs, c_cams = [], [], [], []
         for k in range(n_views):
             xyz, op, feat, scale = flat[4 * k: 4 * k + 4]
             cam = cams[k]
@@ -480,7 +480,8 @@ class _Batch(torch.autograd.Function):
             Dp = torch.empty((H, W), dtype=torch.float32, device=dev)
             v = View()
             v.pts = make_points(xyz, op, feat, scale)
-            v.cam = make_camera(cam)
+            c_cams.append(make_camera(cam))
+            v.cam = c_cams[-1]
             v.out = make_images(F, A, Dp)
             views.append(v)
             outs += [F, A, Dp]
@@ -492,8 +493,9 @@ class _Batch(torch.autograd.Function):
             if st != RAST_OK:
                 raise RastError(st, f"rasterize forward ({stats})")
         # The marshalled options and cameras serve the backward as well: the
-        # pair of passes sees one camera each.
-        ctx.opts, ctx.c_cams, ctx.n_views = opts, [v.cam for v in views], n_views
+        # pair of passes sees one camera each. (The cameras alone: a view's own
+        # camera field would keep the view, with its pointers, alive.)
+        ctx.opts, ctx.c_cams, ctx.n_views = opts, c_cams, n_views
         ctx.save_for_backward(ws, *[t for p in pts for t in p if t is not None])
         ctx.has_scale = [p[3] is not None for p in pts]
         ctx.feat_dtypes = [p[2].dtype for p in pts]
